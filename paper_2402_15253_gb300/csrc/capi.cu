@@ -170,7 +170,7 @@ int launch_single(const Off *rp, const int32_t *ci, int64_t n, int64_t m, int32_
     }
 }
 
-// Validates one graph (see pico_validate_graph): two kernels, then the
+// Validates one graph (see pico_validate_graph): its kernels, then the
 // defect word is read back (the stream is synchronised).
 template <typename Off>
 int validate_impl(const Off *rp, const int32_t *ci, int64_t n, int64_t m, uint32_t *defects,
@@ -188,15 +188,16 @@ int validate_impl(const Off *rp, const int32_t *ci, int64_t n, int64_t m, uint32
     DeviceState *d = nullptr;
     int rc = device_state(&d);
     if (rc != PICO_OK) return rc;
-    unsigned *flag = nullptr;
-    if (fault_alloc() || cudaMallocAsync(&flag, sizeof(unsigned), stream) != cudaSuccess) {
+    pico::ValidateWords *flag = nullptr;
+    if (fault_alloc() || cudaMallocAsync(&flag, sizeof(*flag), stream) != cudaSuccess) {
         cudaGetLastError();
         return PICO_ERR_OOM;
     }
     unsigned found = 0;
-    bool ok = cudaMemsetAsync(flag, 0, sizeof(unsigned), stream) == cudaSuccess &&
+    bool ok = cudaMemsetAsync(flag, 0, sizeof(*flag), stream) == cudaSuccess &&
               pico::launch_validate<Off>(rp, ci, n, m, flag, stream, cfg_of(d)) == 0 &&
-              cudaMemcpyAsync(&found, flag, sizeof(unsigned), cudaMemcpyDeviceToHost, stream) ==
+              cudaMemcpyAsync(&found, &flag->defects, sizeof(unsigned), cudaMemcpyDeviceToHost,
+                              stream) ==
                   cudaSuccess;
     cudaFreeAsync(flag, stream);
     ok = cudaStreamSynchronize(stream) == cudaSuccess && ok;

@@ -132,9 +132,14 @@ int launch_batched(const int64_t *vtx_off, const int64_t *arc_off, int G, const 
 int selftest_wait_timeout(LastResult *last, int limit_ms, cudaStream_t stream, const LaunchCfg &cfg);
 
 // Input validation (validate.cu): ORs the PICO_DEFECT_* bits it finds into
-// *flag (device memory, zeroed by the caller), stream-ordered.
+// words->defects (device memory, zeroed by the caller), stream-ordered.
+struct ValidateWords {
+    unsigned defects;
+    unsigned suspect;    // the quick pass found a defect
+    long long excess;    // ... and how many more arcs it looked up than it skipped
+};
 template <typename Off>
-int launch_validate(const Off *rp, const int *ci, long long n, long long m, unsigned *flag,
+int launch_validate(const Off *rp, const int *ci, long long n, long long m, ValidateWords *words,
                     cudaStream_t stream, const LaunchCfg &cfg);
 
 // The current device's launch configuration and per-device status record
