@@ -1,35 +1,52 @@
-// Batched form: the coreness of G independent graphs in one launch.
+// Batched form: the coreness of G independent graphs.
 //
 // Coreness is defined per connected component (Sec. I: the k-core is a
 // maximal subgraph), so graphs packed side by side are solved independently.
-// The kernel runs the same algorithm bodies as the single-graph kernels
-// (peel::run, histo::run) in two phases over a schedule that lists graphs by
-// decreasing arc count (power-of-two buckets):
-//   large graphs (at least 2^cluster_log2 arcs, a tuning value; listed first): each
-//     thread-block cluster of kClusterCtas CTAs takes one graph at a time
-//     (ClusterDom: counters in the rank-0 CTA's shared memory, reached
-//     through distributed shared memory; hardware cluster barriers);
-//   the rest: every CTA takes one graph at a time (CtaDom: counters in its
-//     own shared memory, __syncthreads).
-// Tickets come from two global counters, so the largest graphs start first
-// and the small ones fill in behind them.
+// A schedule lists the graphs by class, and by decreasing arc count within a
+// class (power-of-two buckets); CTAs and clusters draw tickets from it, so the
+// largest graphs start first and the small ones fill in behind them.
+//
+// PeelOne keeps the residual degrees in shared memory (peel_local.cuh):
+//   tiny    n <= kTinyVertices: CTAs of kTinyThreads threads, eight per SM, so
+//           that one graph's barriers and chains overlap the others'.
+//   middle  n <= kLocalSlots: one CTA of kWideThreads threads per graph.
+//   large   the rest: a cluster of kPeelCtas CTAs per graph; a graph that does
+//           not fit their shared memory either is peeled in global memory
+//           (peel::run over the cluster).
+// Middle and large graphs share one launch: clusters first take the large
+// graphs, then each CTA takes middle ones; the tiny ones are a second launch.
+//
+// HistoCore runs the single-graph body (histo::run) in two phases: graphs of
+// at least 2^cluster_log2 arcs (a tuning value) by clusters of kClusterCtas
+// CTAs (ClusterDom: counters in the rank-0 CTA's shared memory, reached
+// through distributed shared memory; hardware cluster barriers), the rest by
+// one CTA each (CtaDom: counters in its own shared memory, __syncthreads).
 //
 // Scratch is sliced per graph: vertex-indexed arrays at vtx_off[g], the
 // histogram at arc_off[g], and chunk lists at arc_off[g] / 16 + 2g with
 // m_g / 16 + 2 entries (at least m_g / chunk + m_g / (small_deg + 1) + 2 for
 // every allowed tuning: chunk >= 64 and small_deg >= 32).
+#include <algorithm>
+
 #include "histocore.cuh"
+#include "peel_local.cuh"
 #include "peelone.cuh"
+#include "pico.h"
 #include "pico_launch.h"
 
 namespace pico {
 namespace {
 
-constexpr int kBuckets = 64;
-constexpr int kClusterCtas = 8;                 // CTAs per cluster (portable size)
+constexpr int kBuckets = 64;                    // arc-count buckets per class
+constexpr int kClusterCtas = 8;                 // HistoCore: CTAs per cluster (portable size)
+constexpr int kPeelCtas = 4;                    // PeelOne: CTAs per cluster
+constexpr int kWideThreads = 1024;              // PeelOne: threads per CTA of large and middle graphs
+constexpr int kTinyThreads = 128;               // ... and of tiny ones
+constexpr int kTinyVertices = 2048;
 
-// control words of the batched launch (in Ctrl::live)
-enum : int { B_SMALL = 0, B_LARGE = 1, B_NLARGE = 2 };
+// control words of the batched launch (in Ctrl::live): tickets of the classes,
+// the number of graphs in the first class, and in the first two
+enum : int { B_SMALL = 0, B_LARGE = 1, B_NLARGE = 2, B_TINY = 3, B_NMIDDLE = 4 };
 
 struct BatchParams {
     const long long *vtx_off, *arc_off;
@@ -50,40 +67,54 @@ __device__ __forceinline__ int size_bucket(long long m)
     return m <= 0 ? 0 : 64 - __clzll(m);
 }
 
-// Lists the graphs by decreasing arc-count bucket (one CTA) and records how
-// many lead the list with at least 2^cluster_log2 arcs (bucket b holds arc
-// counts in [2^(b-1), 2^b)).
-__global__ void __launch_bounds__(1024)
-    schedule_kernel(const long long *arc_off, int G, int *order, Ctrl *ctl, int cluster_log2)
+// Class of a graph: 2 (listed first) to 0. PeelOne: by where its residual
+// degrees fit; HistoCore: by its arcs (class 1 is not used).
+__device__ __forceinline__ int graph_class(long long n, long long m, int algo, int cluster_log2)
 {
-    __shared__ unsigned cnt[kBuckets];
-    __shared__ unsigned start[kBuckets];
-    if (threadIdx.x < kBuckets) cnt[threadIdx.x] = 0;
+    if (algo != 0) return size_bucket(m) > cluster_log2 ? 2 : 0;
+    return n > peel::kLocalSlots ? 2 : (n > kTinyVertices ? 1 : 0);
+}
+
+// Lists the graphs by class and decreasing arc-count bucket (one CTA) and
+// records how many lead the list in class 2, and in classes 2 and 1 (bucket b
+// holds arc counts in [2^(b-1), 2^b)).
+__global__ void __launch_bounds__(1024)
+    schedule_kernel(const long long *vtx_off, const long long *arc_off, int G, int *order, Ctrl *ctl,
+                    int algo, int cluster_log2)
+{
+    __shared__ unsigned cnt[3 * kBuckets];
+    __shared__ unsigned start[3 * kBuckets];
+    if (threadIdx.x < 3 * kBuckets) cnt[threadIdx.x] = 0;
     __syncthreads();
-    for (int g = threadIdx.x; g < G; g += blockDim.x)
-        atomicAdd(&cnt[size_bucket(arc_off[g + 1] - arc_off[g])], 1u);
+    auto key = [&](int g) {
+        const long long n = vtx_off[g + 1] - vtx_off[g], m = arc_off[g + 1] - arc_off[g];
+        return graph_class(n, m, algo, cluster_log2) * kBuckets + size_bucket(m);
+    };
+    for (int g = threadIdx.x; g < G; g += blockDim.x) atomicAdd(&cnt[key(g)], 1u);
     __syncthreads();
     if (threadIdx.x == 0) {
         unsigned run = 0;
-        for (int b = kBuckets - 1; b >= 0; --b) {
+        for (int b = 3 * kBuckets - 1; b >= 0; --b) {
             start[b] = run;
             run += cnt[b];
-            if (b == cluster_log2 + 1) ctl->live.w[B_NLARGE] = run;
+            if (b == 2 * kBuckets) ctl->live.w[B_NLARGE] = run;
+            if (b == kBuckets) ctl->live.w[B_NMIDDLE] = run;
         }
     }
     __syncthreads();
     for (int g = threadIdx.x; g < G; g += blockDim.x) {
-        const unsigned pos = atomicAdd(&start[size_bucket(arc_off[g + 1] - arc_off[g])], 1u);
+        const unsigned pos = atomicAdd(&start[key(g)], 1u);
         order[pos] = g;
     }
 }
 
-// Solves graph g of the batch in domain `dom`.
+// Solves graph g of the batch in domain `dom`, with its state in global memory.
 template <int Algo, typename Dom>
 __device__ __forceinline__ void solve_graph(const BatchParams &bp, int g, Dom &dom, unsigned *s_tmp,
                                             unsigned long long *st, PhaseClock &clk,
                                             unsigned long long &arcs, unsigned long long &atomics,
-                                            unsigned long long &slots, unsigned long long &pulled)
+                                            unsigned long long &slots, unsigned long long &pulled,
+                                            unsigned long long &extra)
 {
     const long long v0 = bp.vtx_off[g], n = bp.vtx_off[g + 1] - v0;
     const long long a0 = bp.arc_off[g], m = bp.arc_off[g + 1] - a0;
@@ -95,7 +126,6 @@ __device__ __forceinline__ void solve_graph(const BatchParams &bp, int g, Dom &d
         peel::Params<int> p{bp.rp + v0 + g, bp.ci + a0,    n,      bp.core + v0,
                             bp.res0 + v0,   bp.res1 + v0,  bp.qs + v0, chunks,
                             chunk_cap,      bp.ctl,        bp.tn};
-        unsigned long long extra = 0;
         peel::run(p, dom, s_tmp, st, clk, arcs, atomics, extra);
     } else {
         histo::Params<int> p;
@@ -125,9 +155,10 @@ __device__ __forceinline__ void solve_graph(const BatchParams &bp, int g, Dom &d
     }
 }
 
-template <int Algo, int Threads>
+// HistoCore.
+template <int Threads>
 __global__ void __launch_bounds__(Threads, 512 / Threads * 2)
-    batched_kernel(BatchParams bp, LastResult *last)
+    batched_histo_kernel(BatchParams bp, LastResult *last)
 {
     namespace cg = cooperative_groups;
     __shared__ __align__(16) unsigned s_live[kLiveWords];   // 64-bit counters need 8-byte alignment
@@ -141,7 +172,7 @@ __global__ void __launch_bounds__(Threads, 512 / Threads * 2)
     cg::cluster_group cluster = cg::this_cluster();
     const unsigned crank = cluster.block_rank(), csize = cluster.num_blocks();
     PhaseClock clk;
-    unsigned long long arcs = 0, atomics = 0, slots = 0, pulled = 0;
+    unsigned long long arcs = 0, atomics = 0, slots = 0, pulled = 0, extra = 0;
 
     // phase 1: large graphs, one cluster per graph
     const int nlarge = (int)ld_relaxed(&bp.ctl->live.w[B_NLARGE]);
@@ -158,7 +189,7 @@ __global__ void __launch_bounds__(Threads, 512 / Threads * 2)
             const int t = *ticket0;
             cluster.sync();
             if (t < 0) break;
-            solve_graph<Algo>(bp, bp.order[t], dom, s_tmp, st, clk, arcs, atomics, slots, pulled);
+            solve_graph<1>(bp, bp.order[t], dom, s_tmp, st, clk, arcs, atomics, slots, pulled, extra);
         }
     }
     // phase 2: the other graphs, one CTA per graph
@@ -170,7 +201,7 @@ __global__ void __launch_bounds__(Threads, 512 / Threads * 2)
             const int t = s_ticket;
             __syncthreads();
             if (t >= bp.G || status_of(bp.ctl) != 0) break;
-            solve_graph<Algo>(bp, bp.order[t], dom, s_tmp, st, clk, arcs, atomics, slots, pulled);
+            solve_graph<1>(bp, bp.order[t], dom, s_tmp, st, clk, arcs, atomics, slots, pulled, extra);
             __syncthreads();
         }
     }
@@ -178,12 +209,135 @@ __global__ void __launch_bounds__(Threads, 512 / Threads * 2)
     block_sum_to(atomics, &bp.ctl->stats[kStAtomics], s_red);
     block_sum_to(slots, &bp.ctl->stats[kStSlots], s_red);
     block_sum_to(pulled, &bp.ctl->stats[kStPulled], s_red);
-    if (threadIdx.x == 0) {
-        atomicMax(&bp.ctl->stats[kStKmax], st[kStKmax]);
-        st[kStKmax] = 0;
-    }
-    finish_block(bp.ctl, last, Algo, st, kStCount);
+    finish_block(bp.ctl, last, 1, st, kStCount);
     cluster.sync();   // no CTA leaves while another may still read its shared memory
+}
+
+__device__ __forceinline__ peel::LocalParams<int> local_params(const BatchParams &bp, int g)
+{
+    const long long v0 = bp.vtx_off[g], a0 = bp.arc_off[g];
+    return {bp.rp + v0 + g, bp.ci + a0,  (int)(bp.vtx_off[g + 1] - v0), bp.arc_off[g + 1] - a0,
+            bp.core + v0,   bp.qs + v0, bp.ctl};
+}
+
+// PeelOne, large and middle graphs.
+__global__ void __launch_bounds__(kWideThreads, 1) batched_peel_kernel(BatchParams bp)
+{
+    namespace cg = cooperative_groups;
+    extern __shared__ __align__(16) char smem[];
+    __shared__ __align__(16) unsigned s_live[kLiveWords];
+    __shared__ unsigned s_snap[kLiveWords + 1];
+    __shared__ unsigned s_tmp[256];
+    __shared__ unsigned long long s_red[32];
+    __shared__ unsigned long long st[kStCount];
+    __shared__ int s_ticket;
+    if (threadIdx.x < kStCount) st[threadIdx.x] = 0;
+    __syncthreads();
+    cg::cluster_group cluster = cg::this_cluster();
+    const unsigned crank = cluster.block_rank();
+    PhaseClock clk;
+    unsigned long long arcs = 0, atomics = 0, slots = 0, pulled = 0, extra = 0;
+
+    const int nlarge = (int)ld_relaxed(&bp.ctl->live.w[B_NLARGE]);
+    const int nmiddle = (int)ld_relaxed(&bp.ctl->live.w[B_NMIDDLE]);
+    {   // large graphs, one cluster per graph
+        ClusterDom dom{bp.ctl, s_live, cluster.map_shared_rank(s_live, 0), s_snap, crank, kPeelCtas,
+                       0u};
+        int *ticket0 = cluster.map_shared_rank(&s_ticket, 0);
+        for (;;) {
+            if (crank == 0 && threadIdx.x == 0) {
+                const int t = (int)atomicAdd(&bp.ctl->live.w[B_LARGE], 1u);
+                s_ticket = (t < nlarge && status_of(bp.ctl) == 0) ? t : -1;
+            }
+            cluster.sync();
+            const int t = *ticket0;
+            cluster.sync();
+            if (t < 0) break;
+            const int g = bp.order[t];
+            if (bp.vtx_off[g + 1] - bp.vtx_off[g] <= (long long)kPeelCtas * peel::kLocalSlots) {
+                const peel::LocalParams<int> p = local_params(bp, g);
+                const peel::LocalStats s =
+                    peel::run_local<int, peel::LocalWide, true>(p, smem, crank, kPeelCtas);
+                if (crank == 0 && threadIdx.x == 0) peel::add_stats(st, s, p.n, p.m);
+            } else {
+                solve_graph<0>(bp, g, dom, s_tmp, st, clk, arcs, atomics, slots, pulled, extra);
+            }
+        }
+    }
+    for (;;) {   // middle graphs, one CTA per graph
+        if (threadIdx.x == 0) s_ticket = nlarge + (int)atomicAdd(&bp.ctl->live.w[B_SMALL], 1u);
+        __syncthreads();
+        const int t = s_ticket;
+        __syncthreads();
+        if (t >= nmiddle || status_of(bp.ctl) != 0) break;
+        const peel::LocalParams<int> p = local_params(bp, bp.order[t]);
+        const peel::LocalStats s = peel::run_local<int, peel::LocalWide, false>(p, smem, 0, 1);
+        if (threadIdx.x == 0) peel::add_stats(st, s, p.n, p.m);
+        __syncthreads();
+    }
+    block_sum_to(arcs, &bp.ctl->stats[kStArcs], s_red);
+    block_sum_to(atomics, &bp.ctl->stats[kStAtomics], s_red);
+    block_sum_to(extra, &bp.ctl->stats[kStExtra], s_red);
+    fold_block(bp.ctl, st);
+    cluster.sync();   // no CTA leaves while another may still read its shared memory
+}
+
+// PeelOne, tiny graphs; the second launch of a batch, which publishes its
+// status and statistics.
+__global__ void __launch_bounds__(kTinyThreads, 8) batched_tiny_kernel(BatchParams bp, LastResult *last)
+{
+    extern __shared__ __align__(16) char smem[];
+    __shared__ unsigned long long st[kStCount];
+    __shared__ int s_ticket;
+    if (threadIdx.x < kStCount) st[threadIdx.x] = 0;
+    __syncthreads();
+    const int nmiddle = (int)ld_relaxed(&bp.ctl->live.w[B_NMIDDLE]);
+    for (;;) {
+        if (threadIdx.x == 0) s_ticket = nmiddle + (int)atomicAdd(&bp.ctl->live.w[B_TINY], 1u);
+        __syncthreads();
+        const int t = s_ticket;
+        __syncthreads();
+        if (t >= bp.G || status_of(bp.ctl) != 0) break;
+        const peel::LocalParams<int> p = local_params(bp, bp.order[t]);
+        if (p.n <= 0) continue;
+        const peel::LocalStats s = peel::run_local<int, peel::LocalTiny, false>(p, smem, 0, 1);
+        if (threadIdx.x == 0) peel::add_stats(st, s, p.n, p.m);
+        __syncthreads();
+    }
+    fold_kmax(bp.ctl, st);
+    finish_block(bp.ctl, last, PICO_ALGO_PEELONE, st, kStCount);
+}
+
+// Launches a kernel over a persistent grid of clusters: every cluster that is
+// resident at once, but no more than `need`. occ: the kernel's cached number
+// of resident clusters (0: not known yet).
+cudaError_t launch_clusters(const void *fn, int cluster, int threads, size_t smem, int sms,
+                            long long need, int &occ, void **args, cudaStream_t stream)
+{
+    cudaLaunchConfig_t lc = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = cluster;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    lc.blockDim = dim3(threads);
+    lc.dynamicSmemBytes = smem;
+    lc.stream = stream;
+    lc.attrs = attr;
+    lc.numAttrs = 1;
+    if (occ == 0) {
+        if (smem > 0) {
+            const cudaError_t e =
+                cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+        }
+        lc.gridDim = dim3(cluster * sms);
+        const cudaError_t e = cudaOccupancyMaxActiveClusters(&occ, fn, &lc);
+        if (e != cudaSuccess) return e;
+        if (occ <= 0) return cudaErrorLaunchOutOfResources;
+    }
+    lc.gridDim = dim3(cluster * (unsigned)std::min<long long>(need, occ));
+    return cudaLaunchKernelExC(&lc, fn, args);
 }
 
 }  // namespace
@@ -238,37 +392,36 @@ int launch_batched(const int64_t *vtx_off, const int64_t *arc_off, int G, const 
     bp.chunks = c.take<int2>((size_t)(total_m / 16 + 2ll * G + 2));
     bp.tn = cfg.tn;
     if (cudaMemsetAsync(bp.ctl, 0, sizeof(Ctrl), stream) != cudaSuccess) return -3;
-    schedule_kernel<<<1, 1024, 0, stream>>>(bp.arc_off, G, bp.order, bp.ctl, cfg.tn.cluster_log2);
+    schedule_kernel<<<1, 1024, 0, stream>>>(bp.vtx_off, bp.arc_off, G, bp.order, bp.ctl, algo,
+                                            cfg.tn.cluster_log2);
     if (cudaGetLastError() != cudaSuccess) return -3;
 
-    const int threads = cfg.batched_threads == 256 ? 256 : 512;
-    const int vi = (algo & 1) * 2 + (threads == 256 ? 1 : 0);
-    static int occ[4][64] = {};
-    int &o = occ[vi][cfg.device & 63];
-    const void *fns[4] = {(const void *)batched_kernel<0, 512>, (const void *)batched_kernel<0, 256>,
-                          (const void *)batched_kernel<1, 512>, (const void *)batched_kernel<1, 256>};
-    const void *fn = fns[vi];
-    cudaLaunchConfig_t lc = {};
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = kClusterCtas;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    lc.blockDim = dim3(threads);
-    lc.dynamicSmemBytes = 0;
-    lc.stream = stream;
-    lc.attrs = attr;
-    lc.numAttrs = 1;
-    if (o == 0) {   // clusters that fit on the device at once
-        lc.gridDim = dim3(kClusterCtas * cfg.sms);
-        if (cudaOccupancyMaxActiveClusters(&o, fn, &lc) != cudaSuccess || o <= 0) return -3;
+    const int dev = cfg.device & 63;
+    if (algo == 0) {
+        static int occ_wide[64] = {}, occ_tiny[64] = {};
+        void *args[] = {&bp, &last};
+        // graphs the launch can hold (its grids need no more CTAs than that)
+        const long long wide = std::min<long long>(G, total_n / (kTinyVertices + 1));
+        if (wide > 0 &&
+            launch_clusters((const void *)batched_peel_kernel, kPeelCtas, kWideThreads,
+                            peel::local_smem_bytes<peel::LocalWide>(peel::kLocalSlots), cfg.sms,
+                            wide, occ_wide[dev], args, stream) != cudaSuccess)
+            return -3;
+        if (launch_clusters((const void *)batched_tiny_kernel, 1, kTinyThreads,
+                            peel::local_smem_bytes<peel::LocalTiny>(kTinyVertices), cfg.sms * 8, G,
+                            occ_tiny[dev], args, stream) != cudaSuccess)
+            return -3;
+        return 0;
     }
-    // persistent grid: every resident cluster, but no more clusters than graphs need
-    const long long need = ((long long)G + kClusterCtas - 1) / kClusterCtas;
-    const int clusters = need < o ? (int)need : o;
-    lc.gridDim = dim3(kClusterCtas * clusters);
+    static int occ[2][64] = {};
+    const bool narrow = cfg.batched_threads == 256;
     void *args[] = {&bp, &last};
-    if (cudaLaunchKernelExC(&lc, fn, args) != cudaSuccess) return -3;
+    const long long need = ((long long)G + kClusterCtas - 1) / kClusterCtas;
+    if (launch_clusters(narrow ? (const void *)batched_histo_kernel<256>
+                               : (const void *)batched_histo_kernel<512>,
+                        kClusterCtas, narrow ? 256 : 512, 0, cfg.sms, need, occ[narrow][dev], args,
+                        stream) != cudaSuccess)
+        return -3;
     return 0;
 }
 

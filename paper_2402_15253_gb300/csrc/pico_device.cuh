@@ -315,6 +315,27 @@ static __device__ __noinline__ bool grid_sync(Ctrl *c, unsigned *s_snap,
     return grid_sync_hook(c, s_snap, limit_ns, gen, NoHook{});
 }
 
+// Folds the CTA's largest level into the call's control block as a maximum
+// (the other statistics are sums) and clears it in st.
+__device__ __forceinline__ void fold_kmax(Ctrl *c, unsigned long long *st)
+{
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        atomicMax(&c->stats[kStKmax], st[kStKmax]);
+        st[kStKmax] = 0;
+    }
+    __syncthreads();
+}
+
+// The end of a launch that is not the last one of its call: the CTA's
+// statistics go into the control block and nothing is published.
+__device__ __forceinline__ void fold_block(Ctrl *c, unsigned long long *st)
+{
+    fold_kmax(c, st);
+    if (threadIdx.x < kStCount && st[threadIdx.x])
+        atomicAdd(&c->stats[threadIdx.x], st[threadIdx.x]);
+}
+
 // Called once by every CTA at the end of a persistent kernel: folds the CTA's
 // statistics into the call's control block; the last CTA publishes the
 // status and statistics to the per-device LastResult.
@@ -498,8 +519,10 @@ __device__ __forceinline__ unsigned batch_width(unsigned nsmall, unsigned nbig, 
 {
     if (nsmall == 0) return 32u;
     const unsigned free_warps = nwarps > nbig ? nwarps - nbig : 1u;
+    // smallest power of two with at least free_warps units left (one division
+    // instead of one per halving)
     unsigned vb = 32u;
-    while (vb > 1u && (nsmall + vb - 1u) / vb < free_warps) vb >>= 1;
+    while (vb > 1u && nsmall <= vb * (free_warps - 1u)) vb >>= 1;
     return vb;
 }
 
