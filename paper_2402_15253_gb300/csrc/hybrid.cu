@@ -1,6 +1,7 @@
-// Method selection per graph (PICO_ALGO_AUTO): one persistent cooperative
-// kernel that first measures the graph's largest degree, then runs PeelOne or
-// HistoCore on it. The decision is made on the device (no host round trip, so
+// Method selection per graph (PICO_ALGO_AUTO): a persistent cooperative
+// kernel that first measures the graph's largest degree, then runs HistoCore or
+// the first part of PeelOne on it; the launches that follow finish PeelOne, or
+// return at once after HistoCore. The decision is made on the device (no host round trip, so
 // the call stays asynchronous and capturable) and is uniform over the grid
 // (every CTA reads the same snapshot after the barrier).
 //
@@ -37,7 +38,7 @@ __device__ __forceinline__ bool prefer_histocore(long long n, long long m, unsig
 template <typename Off>
 __global__ void __launch_bounds__(kThreads, 2)
     hybrid_kernel(peel::Params<Off> pp, histo::Params<Off> hp, LastResult *last,
-                  unsigned long long limit_ns)
+                  unsigned long long limit_ns, bool local)
 {
     __shared__ unsigned s_snap[kLiveWords + 1];
     __shared__ unsigned s_tmp[256];
@@ -61,25 +62,38 @@ __global__ void __launch_bounds__(kThreads, 2)
          v += (long long)gridDim.x * blockDim.x)
         mx = max(mx, (unsigned)(pp.rp[v + 1] - pp.rp[v]));
     block_max_to(mx, &live[kLiveDmax], s_tmp);
-    bool use_histo = false;
+    bool use_histo = false, over = true;
     if (dom.sync()) {
         if (threadIdx.x == 0) ++st[kStBarriers];
         use_histo = prefer_histocore(n, hp.m, s_snap[kLiveDmax]);
         if (use_histo)
             histo::run(hp, dom, s_tmp, st, clk, arcs, atomics, slots, pulled);
+        else if (local)
+            over = false;   // the next launch peels the graph in shared memory
         else if (pp.work)
-            peel::run_async<Off, kPeelRepair>(pp, dom, s_tmp, st, clk, arcs, atomics, extra);
+            over = peel::run_async<Off, kPeelRepair, true>(pp, dom, s_tmp, st, clk, arcs, atomics,
+                                                           extra, false);
         else
             peel::run<Off, GridDom, kPeelRepair>(pp, dom, s_tmp, st, clk, arcs, atomics, extra);
     }
-    block_sum_to(arcs, &pp.ctl->stats[kStArcs], s_red);
+    if (use_histo || !pp.work) {
+        block_sum_to(arcs, &pp.ctl->stats[kStArcs], s_red);
+    } else if (over && blockIdx.x == 0 && threadIdx.x == 0) {
+        st[kStArcs] = (unsigned long long)hp.m;   // the launch that ends PeelOne counts its arcs
+    }
     block_sum_to(atomics, &pp.ctl->stats[kStAtomics], s_red);
     block_sum_to(slots, &pp.ctl->stats[kStSlots], s_red);
     block_sum_to(pulled, &pp.ctl->stats[kStPulled], s_red);
     block_sum_to(extra, &pp.ctl->stats[kStExtra], s_red);
     if (blockIdx.x != 0 && threadIdx.x < kStCount) st[threadIdx.x] = 0;
-    finish_block(pp.ctl, last, use_histo ? PICO_ALGO_HISTOCORE : PICO_ALGO_PEELONE, st,
-                 kStCount);
+    if (!over) {   // later launches finish and publish
+        fold_block(pp.ctl, st);
+        return;
+    }
+    if (finish_block(pp.ctl, last, use_histo ? PICO_ALGO_HISTOCORE : PICO_ALGO_PEELONE, st,
+                     kStCount) &&
+        pp.work)
+        pp.tail->published = 1;   // the later launches return at once
 }
 
 }  // namespace
@@ -143,13 +157,19 @@ int launch_hybrid(const Off *rp, const int *ci, long long n, long long m, int *c
     }
     if (cudaMemsetAsync(pp.ctl, 0, sizeof(Ctrl), stream) != cudaSuccess) return -3;
     unsigned long long limit = cfg.limit_ns;
-    void *args[] = {&pp, &hp, &last, &limit};
+    bool local = pp.work && peelone_local(n, m);
+    void *args[] = {&pp, &hp, &last, &limit, &local};
     // PeelOne's residual degrees stay in L2 (when HistoCore runs, the window
     // covers part of its scratch instead, which is harmless)
     const size_t win = pp.work ? std::min<size_t>((size_t)n * sizeof(int), cfg.l2_window) : 0;
     if (launch_cooperative((const void *)hybrid_kernel<Off>, dim3(ctas), dim3(kThreads), args, 0,
                            stream, pp.work, win) != cudaSuccess)
         return -3;
+    if (pp.work) {   // what is left of PeelOne, if that is the method
+        const int rc = local ? launch_local(pp, m, pp.tail, last, stream, cfg)
+                             : launch_turns(pp, m, last, stream, cfg, ctas);
+        if (rc != 0) return rc;
+    }
     if (win > 0 && l2_release(pp.work, win, stream) != cudaSuccess) return -3;
     return 0;
 }

@@ -4,6 +4,8 @@
 // levels are switched off.
 #include <algorithm>
 
+#include "peel_local.cuh"
+#include "peel_tail.cuh"
 #include "peelone.cuh"
 #include "pico.h"
 #include "pico_launch.h"
@@ -11,37 +13,175 @@
 namespace pico {
 namespace {
 
-template <typename Off, int Mode, bool kAsync>
+// The shared-memory form: threads of its CTA, and half as many for the
+// smallest graphs, whose waves are a few rows and whose CTA barriers are
+// then cheaper (R-MAT scale 10: 137 against 144 us).
+constexpr int kLocalThreads = 1024;
+constexpr long long kLocalNarrow = 2048;
+// One SM walks about 1.5 arcs per clock, so it loses to the grid where there
+// are many arcs and few levels (Erdos-Renyi, n 50,001, m 0.8 M, 9 levels: 504
+// against 266 us) and wins on skewed graphs up to this size (R-MAT scale 14, m
+// 0.43 M: 545 against 1,503 us; Chung-Lu, n 32,768, m 0.6 M: 794 against 1,229
+// us with the cluster kernel and 2,028 us without).
+constexpr long long kLocalMaxArcs = 640 << 10;
+
+// kTail: one of the launches that alternate with the cluster kernel. The one
+// that ends the run publishes the status and the statistics (the `final` one
+// ends it in any case); the launches after it return at once.
+template <typename Off, int Mode, bool kAsync, bool kTail>
 __global__ void __launch_bounds__(kThreads, 2)
-    peelone_kernel(peel::Params<Off> p, LastResult *last, unsigned long long limit_ns)
+    peelone_kernel(peel::Params<Off> p, LastResult *last, unsigned long long limit_ns,
+                   long long m, bool final)
 {
     __shared__ unsigned s_snap[kLiveWords + 1];
     __shared__ unsigned s_tmp[128];
     __shared__ unsigned long long s_red[32];
     __shared__ unsigned long long st[kStCount];   // statistics, written by thread 0
+    if (kTail && p.tail->published) return;   // the same in every CTA
     if (threadIdx.x < kStCount) st[threadIdx.x] = 0;
     __syncthreads();
     unsigned long long arcs = 0, atomics = 0, extra = 0;
     PhaseClock clk;
     if (blockIdx.x == 0 && threadIdx.x == 0 && last->trace_on) {
-        last->trace_len = 0;
+        if (!kTail || p.tail->mode == peel::kTailFresh) last->trace_len = 0;
         clk.trace = last->trace;
         clk.trace_len = &last->trace_len;
     }
     clk.start();
     GridDom dom{p.ctl, s_snap, limit_ns};
+    bool over = true;
     if (kAsync)
-        peel::run_async<Off, Mode>(p, dom, s_tmp, st, clk, arcs, atomics, extra);
+        over = peel::run_async<Off, Mode, kTail>(p, dom, s_tmp, st, clk, arcs, atomics, extra, final);
     else
         peel::run<Off, GridDom, Mode>(p, dom, s_tmp, st, clk, arcs, atomics, extra);
-    block_sum_to(arcs, &p.ctl->stats[kStArcs], s_red);
+    if (kTail) {   // every row is expanded once, by one kernel or the other
+        if (over && threadIdx.x == 0) st[kStArcs] = (unsigned long long)m;
+    } else {
+        block_sum_to(arcs, &p.ctl->stats[kStArcs], s_red);
+    }
     block_sum_to(atomics, &p.ctl->stats[kStAtomics], s_red);
     block_sum_to(extra, &p.ctl->stats[kStExtra], s_red);
     if (blockIdx.x != 0 && threadIdx.x < kStCount) st[threadIdx.x] = 0;
-    finish_block(p.ctl, last,
-                 Mode == kPeelRepair ? PICO_ALGO_PEELONE
-                                     : (Mode == kPeelCas ? PICO_ALGO_PEEL_CAS : PICO_ALGO_PEEL_ADDBACK),
-                 st, kStCount);
+    if (!over) {
+        fold_block(p.ctl, st);
+        return;
+    }
+    if (kTail) fold_kmax(p.ctl, st);
+    const bool published = finish_block(
+        p.ctl, last,
+        Mode == kPeelRepair ? PICO_ALGO_PEELONE
+                            : (Mode == kPeelCas ? PICO_ALGO_PEEL_CAS : PICO_ALGO_PEEL_ADDBACK),
+        st, kStCount);
+    if (kTail && published) p.tail->published = 1;
+}
+
+// The light levels of a graph on one cluster, between two launches of the grid
+// kernel (peel_tail.cuh).
+template <typename Off>
+__global__ void __launch_bounds__(peel::kTailThreads, 1)
+    peelone_tail_kernel(peel::Params<Off> p, LastResult *last, long long m, bool final)
+{
+    extern __shared__ __align__(16) char smem[];
+    __shared__ unsigned long long st[kStCount];
+    __shared__ unsigned long long s_red[32];
+    // nothing to do (the same in every CTA)
+    if (p.tail->published) return;
+    const bool failed = status_of(p.ctl) != 0;
+    if (!final && (p.tail->mode != peel::kTailScan || failed)) return;
+    if (threadIdx.x < kStCount) st[threadIdx.x] = 0;
+    PhaseClock clk;
+    if (blockIdx.x == 0 && threadIdx.x == 0 && last->trace_on) {
+        clk.trace = last->trace;
+        clk.trace_len = &last->trace_len;
+    }
+    __syncthreads();
+    clk.start();
+    peel::TailPeel<Off> tp{p, p.tail, *reinterpret_cast<peel::TailShared *>(smem), blockIdx.x,
+                            final};
+    const bool over = failed || tp.run(st);
+    if (over && blockIdx.x == 0 && threadIdx.x == 0) st[kStArcs] = (unsigned long long)m;
+    clk.end(st, kPhWaveMid, (unsigned)st[kStLevels]);
+    block_sum_to(tp.n_lowered, &p.ctl->stats[kStAtomics], s_red);
+    if (over) {   // only CTA 0 counts levels and scans
+        fold_kmax(p.ctl, st);
+        if (finish_block(p.ctl, last, PICO_ALGO_PEELONE, st, kStCount)) p.tail->published = 1;
+    } else {
+        fold_block(p.ctl, st);
+    }
+    cooperative_groups::this_cluster().sync();   // no CTA leaves while another may write to it
+}
+
+// A graph whose residual degrees fit the shared memory of one CTA
+// (peel_local.cuh). tail: another launch may have solved it already (nullptr:
+// none has).
+template <typename Off>
+__global__ void __launch_bounds__(kLocalThreads, 1)
+    peelone_local_kernel(peel::LocalParams<Off> p, const peel::TailState *tail, LastResult *last)
+{
+    extern __shared__ __align__(16) char smem[];
+    __shared__ unsigned long long st[kStCount];
+    if (tail && tail->published) return;
+    if (threadIdx.x < kStCount) st[threadIdx.x] = 0;
+    PhaseClock clk;
+    if (threadIdx.x == 0 && last->trace_on) {
+        last->trace_len = 0;
+        clk.trace = last->trace;
+        clk.trace_len = &last->trace_len;
+    }
+    __syncthreads();
+    clk.start();
+    const peel::LocalStats s = peel::run_local<Off, peel::LocalWide, false>(p, smem, 0, 1);
+    if (threadIdx.x == 0) peel::add_stats(st, s, p.n, p.m);
+    clk.end(st, kPhWaveMid, (unsigned)s.waves);
+    finish_block(p.ctl, last, PICO_ALGO_PEELONE, st, kStCount);
+}
+
+// Sets a kernel's dynamic shared memory limit (and non-portable cluster size)
+// once per device.
+bool prepare_kernel(const void *fn, size_t smem, bool wide_cluster, bool &ready)
+{
+    if (ready) return true;
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+        cudaSuccess)
+        return false;
+    if (wide_cluster &&
+        cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+        return false;
+    ready = true;
+    return true;
+}
+
+template <typename Off>
+cudaError_t launch_tail(peel::Params<Off> &p, long long m, LastResult *last, cudaStream_t stream,
+                        int device, bool final)
+{
+    static bool ready[64] = {};
+    const void *fn = (const void *)peelone_tail_kernel<Off>;
+    constexpr size_t smem = sizeof(peel::TailShared);
+    if (!prepare_kernel(fn, smem, true, ready[device & 63])) return cudaErrorInvalidValue;
+    cudaLaunchConfig_t lc = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = peel::kTailCtas;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    lc.gridDim = dim3(peel::kTailCtas);
+    lc.blockDim = dim3(peel::kTailThreads);
+    lc.dynamicSmemBytes = smem;
+    lc.stream = stream;
+    lc.attrs = attr;
+    lc.numAttrs = 1;
+    void *args[] = {&p, &last, &m, &final};
+    return cudaLaunchKernelExC(&lc, fn, args);
+}
+
+// Launches that follow the grid kernel's first: cluster and grid kernel in turn.
+// A launch with nothing to do takes 4 to 5 us, so small graphs get few and end
+// with the cluster kernel (which walks 5 M arcs at worst in 0.4 ms); large ones
+// end with the grid kernel.
+int tail_launches(long long m)
+{
+    return m < (6 << 20) ? 1 : m < (12 << 20) ? 3 : m < (20 << 20) ? 4 : m < (32 << 20) ? 6 : 12;
 }
 
 // Reads a range (16 bytes a thread per step); the values are not used.
@@ -91,19 +231,83 @@ size_t peelone_ws_bytes(long long n, long long m, bool async)
     return c.size();
 }
 
+bool peelone_local(long long n, long long m)
+{
+    return n <= peel::kLocalSlots && m <= kLocalMaxArcs;
+}
+
+template <typename Off>
+int launch_local(const peel::Params<Off> &p, long long m, const peel::TailState *tail,
+                 LastResult *last, cudaStream_t stream, const LaunchCfg &cfg)
+{
+    static bool ready[64] = {};
+    const void *fn = (const void *)peelone_local_kernel<Off>;
+    if (!prepare_kernel(fn, peel::local_smem_bytes<peel::LocalWide>(peel::kLocalSlots), false,
+                        ready[cfg.device & 63]))
+        return -3;
+    peel::LocalParams<Off> lp{p.rp, p.ci, (int)p.n, m, p.core, p.qs, p.ctl};
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3(1);
+    lc.blockDim = dim3(p.n <= kLocalNarrow ? kLocalThreads / 2 : kLocalThreads);
+    lc.dynamicSmemBytes = peel::local_smem_bytes<peel::LocalWide>((int)p.n);
+    lc.stream = stream;
+    void *args[] = {&lp, &tail, &last};
+    return cudaLaunchKernelExC(&lc, fn, args) == cudaSuccess ? 0 : -3;
+}
+
+template <typename Off>
+int launch_turns(const peel::Params<Off> &p0, long long m, LastResult *last, cudaStream_t stream,
+                 const LaunchCfg &cfg, int ctas)
+{
+    peel::Params<Off> p = p0;
+    unsigned long long limit = cfg.limit_ns;
+    const int launches = tail_launches(m);
+    const size_t win = std::min<size_t>((size_t)p.n * sizeof(int), cfg.l2_window);
+    for (int i = 0; i < launches; ++i) {
+        bool final = i + 1 == launches;
+        void *args[] = {&p, &last, &limit, &m, &final};
+        const cudaError_t e =
+            i % 2 == 0 ? launch_tail(p, m, last, stream, cfg.device, final)
+                       : launch_cooperative((const void *)peelone_kernel<Off, kPeelRepair, true, true>,
+                                            dim3(ctas), dim3(kThreads), args, 0, stream, p.work, win);
+        if (e != cudaSuccess) return -3;
+    }
+    return 0;
+}
+
+template int launch_local<int>(const peel::Params<int> &, long long, const peel::TailState *,
+                               LastResult *, cudaStream_t, const LaunchCfg &);
+template int launch_local<long long>(const peel::Params<long long> &, long long,
+                                     const peel::TailState *, LastResult *, cudaStream_t,
+                                     const LaunchCfg &);
+template int launch_turns<int>(const peel::Params<int> &, long long, LastResult *, cudaStream_t,
+                               const LaunchCfg &, int);
+template int launch_turns<long long>(const peel::Params<long long> &, long long, LastResult *,
+                                     cudaStream_t, const LaunchCfg &, int);
+
 template <typename Off>
 int launch_peelone(const Off *rp, const int *ci, long long n, long long m, int *core, void *ws,
                    LastResult *last, cudaStream_t stream, const LaunchCfg &cfg, int mode)
 {
     if (mode < kPeelRepair || mode > kPeelAddBack) return -1;
-    const void *fns[2][3] = {{(const void *)peelone_kernel<Off, kPeelRepair, false>,
-                              (const void *)peelone_kernel<Off, kPeelCas, false>,
-                              (const void *)peelone_kernel<Off, kPeelAddBack, false>},
-                             {(const void *)peelone_kernel<Off, kPeelRepair, true>,
-                              (const void *)peelone_kernel<Off, kPeelCas, true>,
-                              (const void *)peelone_kernel<Off, kPeelAddBack, true>}};
+    const void *fns[2][3] = {{(const void *)peelone_kernel<Off, kPeelRepair, false, false>,
+                              (const void *)peelone_kernel<Off, kPeelCas, false, false>,
+                              (const void *)peelone_kernel<Off, kPeelAddBack, false, false>},
+                             {(const void *)peelone_kernel<Off, kPeelRepair, true, true>,
+                              (const void *)peelone_kernel<Off, kPeelCas, true, false>,
+                              (const void *)peelone_kernel<Off, kPeelAddBack, true, false>}};
     static int occ[2][3][64] = {};
     bool async = cfg.peel_async;
+    if (async && mode == kPeelRepair && peelone_local(n, m)) {
+        Carver c(ws);
+        peel::Params<Off> p;
+        peel::carve(p, c, n, m, true);
+        p.rp = rp;
+        p.ci = ci;
+        p.core = core;
+        if (cudaMemsetAsync(p.ctl, 0, sizeof(Ctrl), stream) != cudaSuccess) return -3;
+        return launch_local(p, m, nullptr, last, stream, cfg);
+    }
     int &o = occ[async][mode][cfg.device & 63];
     if (o == 0) {
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, fns[async][mode], kThreads, 0) !=
@@ -126,12 +330,15 @@ int launch_peelone(const Off *rp, const int *ci, long long n, long long m, int *
 
     dim3 grid(ctas), block(kThreads);
     unsigned long long limit = cfg.limit_ns;
-    void *args[] = {&p, &last, &limit};
+    const bool tail = async && mode == kPeelRepair;
+    bool final = !tail;
+    void *args[] = {&p, &last, &limit, &m, &final};
     // the residual degrees (the target of every decrement) stay in L2
     const size_t win = async ? std::min<size_t>((size_t)n * sizeof(int), cfg.l2_window) : 0;
     if (launch_cooperative(fns[async][mode], grid, block, args, 0, stream, p.work, win) !=
         cudaSuccess)
         return -3;
+    if (tail && launch_turns(p, m, last, stream, cfg, ctas) != 0) return -3;
     if (win > 0 && l2_release(p.work, win, stream) != cudaSuccess) return -3;
     return 0;
 }

@@ -54,10 +54,47 @@ namespace peel {
 // then (asynchronous levels) the static frontier's small and chunk counts
 enum : int {
     L_QS = 0, L_QB = 1, L_KEPT = 2 /* 2..4 */, L_MIN = 5 /* 5..7 */, L_FS = 8 /* 8..10 */,
-    L_FB = 11 /* 11..13 */
+    L_FB = 11 /* 11..13 */, L_FA = 14 /* 14..16: the static frontier's arcs, capped per warp */, L_DMAX = 17
 };
 
 constexpr int kScanItems = 4;   // residual-list entries per thread per scan step
+
+// Asynchronous levels: a warp that holds dynamic frontier vertices with fewer
+// arcs than this in all walks them without listing any as chunks.
+constexpr unsigned kWalkAtOnce = 512;
+
+// Where a run that alternates between the grid kernel (run_async) and the
+// cluster kernel (peel_tail.cuh) stands. Part of the control block, which is
+// zeroed before the run.
+enum : int {
+    kTailFresh = 0,     // nothing done yet
+    kTailScan = 1,      // the scan of level k comes next, residual list of nres entries
+    kTailPending = 2,   // level k: fs[lo, hi) are queued and not walked
+    kTailDone = 3
+};
+struct TailState {
+    int mode;
+    int k;
+    unsigned nres;      // residual list: may hold vertices queued since it was written
+    unsigned cur;       // ... in res1 (1) or res0
+    unsigned lo, hi;
+    unsigned spilled;   // cluster kernel: entries listed in fs during a wave
+    int skewed;         // the grid kernel may hand levels over
+    int published;      // the run's status and statistics are out (method selection)
+};
+
+// When the grid kernel hands a level over, and the cluster kernel a wave back.
+// The grid takes 17 us for a level with next to no arcs and 20 us more for
+// 0.5 M; the cluster's levels start at 6 us and walk 0.2 M arcs in 20 us. Its
+// first scan reads the whole residual list (0.5 M vertices: 30 us). A graph
+// without skew has few levels, most of them heavy: handing over its two or
+// three light ones costs more than it saves (Erdos-Renyi, n 300,007, m 4.8 M:
+// 344 us without, 459 us with).
+constexpr unsigned kTailMaxResidual = 512u << 10;
+constexpr unsigned kTailMaxArcs = 64u << 10;
+constexpr unsigned kTailBudget = 128u << 10;
+static_assert(sizeof(TailState) <= sizeof(Line), "the control block has no room for TailState");
+constexpr long long kTailSkew = 16;   // largest degree at least this many times the mean
 
 template <typename Off>
 struct Params {
@@ -76,6 +113,7 @@ struct Params {
     int *fs = nullptr;    // the scan's frontier of small vertices, n slots
     int2 *fb = nullptr;   // the scan's frontier chunk entries, qb_cap slots
     Line *actl = nullptr; // AsyncLine lines, then one line per CTA (level-end flags)
+    TailState *tail = nullptr;   // state shared with the cluster kernel (nullptr: none)
 };
 
 // Lines of the asynchronous level control block (run_async).
@@ -107,11 +145,13 @@ inline void carve(Params<Off> &p, C &c, long long n, long long m, bool async)
         p.fs = c.template take<int>(n);
         p.fb = c.template take<int2>(p.qb_cap);
         p.actl = c.template take<Line>(A_FLAGS + kMaxAsyncCtas);
+        p.tail = reinterpret_cast<TailState *>(p.ctl->tail.w);
     } else {
         p.work = nullptr;
         p.fs = nullptr;
         p.fb = nullptr;
         p.actl = nullptr;
+        p.tail = nullptr;
     }
 }
 
@@ -419,37 +459,44 @@ __device__ __forceinline__ bool hub_guard(long long d, int k, int g)
     return g > 0 && d > (long long)g * k;
 }
 
+// Arc ranges of the lane's row (first arc rs, d arcs): the c-th one is
+// [a, b), written as (a, b), or as (a, ~b) when `guard` is set (b >= 1, so ~b
+// <= -2 never equals the empty slot's -1).
+struct RangeEntry {
+    int rs, d, chunk;
+    bool guard;
+    mutable int rs2 = 0, d2 = 0;
+    mutable bool guard2 = false;
+    __device__ __forceinline__ RangeEntry(int s, int n, int size, bool g)
+        : rs(s), d(n), chunk(size), guard(g) {}
+    __device__ __forceinline__ void take(int src) const
+    {
+        rs2 = __shfl_sync(kFull, rs, src);
+        d2 = __shfl_sync(kFull, d, src);
+        guard2 = __shfl_sync(kFull, (int)guard, src) != 0;
+    }
+    __device__ __forceinline__ int2 operator()(int lane, unsigned c) const
+    {
+        const int s = lane >= 0 ? rs : rs2, n = lane >= 0 ? d : d2;
+        const int a = s + (int)c * chunk, b = n - (int)c * chunk > chunk ? a + chunk : s + n;
+        return make_int2(a, (lane >= 0 ? guard : guard2) ? ~b : b);
+    }
+};
+
 // Warp-cooperative append of the arc ranges of large vertices: every lane
-// with `pred` owns a vertex whose row starts at rs and holds d arcs; the warp
-// writes the ceil(d / chunk) ranges [a, b) of each such vertex in turn, as
-// (a, b), or as (a, ~b) when `guard` is set (b >= 1, so ~b <= -2 never
-// equals the empty slot's -1).
+// with `pred` owns a vertex whose row starts at rs and holds d arcs.
 __device__ __forceinline__ void warp_push_ranges(bool pred, int rs, int d, bool guard, int2 *list,
                                                  unsigned *counter, unsigned cap, Ctrl *ctl,
                                                  int chunk)
 {
-    const int lane = threadIdx.x & 31;
-    unsigned m = __ballot_sync(kFull, pred);
-    while (m) {
-        const int src = __ffs(m) - 1;
-        m &= m - 1;
-        const int s0 = __shfl_sync(kFull, rs, src);
-        const int dd = __shfl_sync(kFull, d, src);
-        const bool gg = __shfl_sync(kFull, (int)guard, src) != 0;
-        const unsigned nch = (unsigned)((dd + chunk - 1) / chunk);
-        unsigned pos = 0;
-        if (lane == 0) pos = atomicAdd(counter, nch);
-        pos = __shfl_sync(kFull, pos, 0);
-        if ((unsigned long long)pos + nch > cap) {
-            if (lane == 0) set_error(ctl, kErrNotConverged);
-            continue;
-        }
-        for (unsigned c = lane; c < nch; c += 32) {
-            const int a = s0 + (int)c * chunk;
-            const int b = dd - (int)c * chunk > chunk ? a + chunk : s0 + dd;
-            st_relaxed(list + pos + c, make_int2(a, gg ? ~b : b));
-        }
+    unsigned nch = pred ? (unsigned)((d + chunk - 1) / chunk) : 0u;
+    const unsigned pos = warp_reserve(counter, nch);
+    if (nch > 0 && (unsigned long long)pos + nch > cap) {
+        set_error(ctl, kErrNotConverged);
+        nch = 0;
     }
+    if (__any_sync(kFull, nch > 0))
+        warp_fill<true>(nch, pos, list, RangeEntry(rs, d, chunk, guard));
 }
 
 // One warp walks the arcs [s, t) of col_idx (a range entry).
@@ -561,10 +608,14 @@ __device__ __forceinline__ void walk_chunk_guarded(const Off *__restrict__ rp,
 // the result; each vertex is still queued exactly once (one decrement takes
 // it from k + 1 to k, or the scan finds it at k), so the levels, the arcs
 // walked and the successful decrements are the same as in the wave form.
-template <typename Off, int Mode = kPeelRepair>
-__device__ void run_async(const Params<Off> &p, GridDom &dom, unsigned *s_tmp,
+//
+// kTail: the run alternates with the cluster kernel of peel_tail.cuh. It starts
+// from *p.tail and, unless `last`, leaves before the walk of a light level; it
+// returns false then (the same in every thread), true when the run is over.
+template <typename Off, int Mode = kPeelRepair, bool kTail = false>
+__device__ bool run_async(const Params<Off> &p, GridDom &dom, unsigned *s_tmp,
                           unsigned long long *st, PhaseClock &clk, unsigned long long &arcs,
-                          unsigned long long &atomics, unsigned long long &extra)
+                          unsigned long long &atomics, unsigned long long &extra, bool last = true)
 {
     Ctrl *ctl = p.ctl;
     unsigned *live = dom.live();
@@ -584,10 +635,12 @@ __device__ void run_async(const Params<Off> &p, GridDom &dom, unsigned *s_tmp,
     __shared__ unsigned s_busy;                // warps of this CTA that are not idle
     __shared__ unsigned long long s_acc;       // walked by idle warps, not yet in `done`
 
+    const int mode = kTail ? ld_relaxed(&p.tail->mode) : (int)kTailFresh;
+    if (kTail && (mode == kTailDone || status_of(ctl) != 0)) return true;
     // init: work = degree, isolated vertices get 0, residual list, queue
     // slots empty, control lines zero
-    {
-        unsigned mx = 0;
+    if (mode == kTailFresh) {
+        unsigned mx = 0, dmax = 0;
         for (long long base = first; base < n; base += nthreads) {
             const long long v = base + threadIdx.x;
             bool keep = false;
@@ -598,6 +651,7 @@ __device__ void run_async(const Params<Off> &p, GridDom &dom, unsigned *s_tmp,
                 p.qs[v] = -1;
                 keep = d > 0;
                 if (keep) mx = max(mx, (unsigned)(INT_MAX - d));
+                if (kTail) dmax = max(dmax, (unsigned)d);
             }
             unsigned pos, unused;
             block_push2(keep, false, &live[L_KEPT], &live[L_KEPT], pos, unused, s_tmp);
@@ -608,37 +662,72 @@ __device__ void run_async(const Params<Off> &p, GridDom &dom, unsigned *s_tmp,
         if (blockIdx.x == 0 && threadIdx.x < 32 * A_FLAGS)
             p.actl[threadIdx.x >> 5].w[threadIdx.x & 31] = 0;
         block_max_to(mx, &live[L_MIN], s_tmp);
+        if (kTail) block_max_to(dmax, &live[L_DMAX], s_tmp);
+        if (!dom.sync()) return true;
+        if (threadIdx.x == 0) ++st[kStBarriers];
+        clk.end(st, kPhInit);
     }
-    if (!dom.sync()) return;
-    if (threadIdx.x == 0) ++st[kStBarriers];
-    clk.end(st, kPhInit);
 
-    unsigned nres = snap[L_KEPT];
-    int k = INT_MAX - (int)snap[L_MIN];
+    unsigned nres;
+    int k;
     unsigned slot = 1;   // kept/min/frontier slot of the next scan (slot 0: init)
     int cur = 0;
     unsigned long long listed_static = 0;   // scan frontier entries of all levels so far
+    bool pending = false;                   // the level's first vertices are listed already
+    bool skewed = true;
+    if (mode == kTailFresh) {
+        nres = snap[L_KEPT];
+        k = INT_MAX - (int)snap[L_MIN];
+        if (kTail) skewed = (long long)snap[L_DMAX] * n >= kTailSkew * (long long)p.rp[n];
+    } else {
+        nres = p.tail->nres;
+        k = p.tail->k;
+        cur = (int)p.tail->cur;
+        pending = mode == kTailPending;
+        // everything listed in earlier launches has been walked
+        listed_static = __ldcg(done) - (unsigned long long)ld_relaxed(&live[L_QS]) -
+                        (unsigned long long)ld_relaxed(&live[L_QB]);
+    }
     long long scans = 0;
     const long long max_scans = 2 * n + 4;
     const unsigned long long limit_ns = dom.limit_ns;
 
-    while (nres > 0) {
+    const auto set_heads = [&](const uint4 *t) {
+        const unsigned *w = reinterpret_cast<const unsigned *>(t);
+        __stcg(qs_head, w[L_QS] + 32u * nwarps);
+        __stcg(qb_head, w[L_QB] + nwarps);
+    };
+    while (nres > 0 || pending) {
         if (++scans > max_scans) {
             if (threadIdx.x == 0) set_error(ctl, kErrNotConverged);
-            return;
+            return true;
         }
+        unsigned t0, b0, nfs, nfb;
+        const bool resumed = pending;
+        if (resumed) {   // the cluster kernel's queue
+            pending = false;
+            if (!dom.sync_hook(set_heads)) return true;
+            if (threadIdx.x == 0) ++st[kStBarriers];
+            clk.end(st, kPhInit);
+            t0 = snap[L_QS];
+            b0 = snap[L_QB];
+            nfs = p.tail->hi - p.tail->lo;
+            nfb = 0;
+        } else {
         if (dom.leader()) {
             const unsigned nx = (slot + 1) % 3;
             live[L_KEPT + nx] = 0;
             live[L_MIN + nx] = 0;
             live[L_FS + nx] = 0;
             live[L_FB + nx] = 0;
+            live[L_FA + nx] = 0;
         }
 
         // scan the residual list at level k (kScanItems vertices per thread)
         const int *rin = cur ? p.res1 : p.res0;
         int *rout = cur ? p.res0 : p.res1;
         unsigned mx = 0;
+        unsigned long long front_arcs = 0;
         const long long step = (long long)nthreads * kScanItems;
         for (long long base = first * kScanItems; base < nres; base += step) {
             int v[kScanItems], c[kScanItems];
@@ -657,6 +746,7 @@ __device__ void run_async(const Params<Off> &p, GridDom &dom, unsigned *s_tmp,
                 if (c[j] == k) {
                     d[j] = (long long)(p.rp[v[j] + 1] - p.rp[v[j]]);
                     p.core[v[j]] = k;
+                    if (kTail) front_arcs += (unsigned long long)d[j];
                 }
                 nsmall += (c[j] == k && d[j] <= p.tn.small_deg);
                 nkeep += (c[j] > k);
@@ -674,15 +764,15 @@ __device__ void run_async(const Params<Off> &p, GridDom &dom, unsigned *s_tmp,
                 warp_push_chunks(c[j] == k && d[j] > p.tn.small_deg, v[j], d[j], p.fb,
                                  &live[L_FB + slot], p.qb_cap, ctl, p.tn.chunk);
         }
+        if (kTail && !last) {   // rare: most threads find no vertex at k
+            const unsigned a = (unsigned)min(front_arcs, 1ull << 18);
+            const unsigned sum = __reduce_add_sync(kFull, a);
+            if (lane == 0 && sum) atomicAdd(&live[L_FA + slot], min(sum, 1u << 18));
+        }
         block_max_to(mx, &live[L_MIN + slot], s_tmp);
         // the last arrival deals out the level's first tickets by moving the
         // heads past them
-        const bool ok = dom.sync_hook([&](const uint4 *t) {
-            const unsigned *w = reinterpret_cast<const unsigned *>(t);
-            __stcg(qs_head, w[L_QS] + 32u * nwarps);
-            __stcg(qb_head, w[L_QB] + nwarps);
-        });
-        if (!ok) return;
+        if (!dom.sync_hook(set_heads)) return true;
         if (threadIdx.x == 0) {
             ++st[kStBarriers];
             ++st[kStScans];
@@ -690,8 +780,20 @@ __device__ void run_async(const Params<Off> &p, GridDom &dom, unsigned *s_tmp,
         }
         clk.end(st, kPhScan, nres);
 
-        const unsigned t0 = snap[L_QS], b0 = snap[L_QB];
-        const unsigned nfs = snap[L_FS + slot], nfb = snap[L_FB + slot];
+        t0 = snap[L_QS];
+        b0 = snap[L_QB];
+        nfs = snap[L_FS + slot];
+        nfb = snap[L_FB + slot];
+        if (kTail && !last && skewed &&
+            nres <= kTailMaxResidual && snap[L_FA + slot] <= kTailMaxArcs) {
+            if (dom.leader()) {   // the level is light: the cluster kernel scans it again
+                p.tail->mode = kTailScan;
+                p.tail->k = k;
+                p.tail->nres = nres;
+                p.tail->cur = (unsigned)cur;
+            }
+            return false;
+        }
         nres = snap[L_KEPT + slot];
         const int kmin_kept = INT_MAX - (int)snap[L_MIN + slot];
         slot = (slot + 1) % 3;
@@ -703,6 +805,7 @@ __device__ void run_async(const Params<Off> &p, GridDom &dom, unsigned *s_tmp,
         if (threadIdx.x == 0) {
             ++st[kStLevels];
             if ((unsigned long long)k > st[kStKmax]) st[kStKmax] = (unsigned long long)k;
+        }
         }
         listed_static += nfs + nfb;
 
@@ -724,12 +827,20 @@ __device__ void run_async(const Params<Off> &p, GridDom &dom, unsigned *s_tmp,
                 rs = p.rp[v];
                 d = (long long)(p.rp[v + 1] - rs);
             }
-            const bool large = d > p.tn.small_deg;
-            if (RangeEntries<Off>::value)
-                warp_push_ranges(large, (int)rs, (int)d, hub_guard(d, k, p.tn.peel_guard), p.qb,
-                                 &live[L_QB], p.qb_cap, ctl, p.tn.chunk);
-            else
-                warp_push_chunks<true>(large, v, d, p.qb, &live[L_QB], p.qb_cap, ctl, p.tn.chunk);
+            bool large = d > p.tn.small_deg;
+            if (__any_sync(kFull, large)) {
+                // a warp whose rows hold few arcs walks them at once, whatever
+                // their degrees: handing them over costs an append, a poll and a
+                // pick-up
+                const unsigned sum = __reduce_add_sync(
+                    kFull, (unsigned)(d < (long long)kWalkAtOnce ? d : (long long)kWalkAtOnce));
+                large = large && sum >= kWalkAtOnce;
+                if (RangeEntries<Off>::value)
+                    warp_push_ranges(large, (int)rs, (int)d, hub_guard(d, k, p.tn.peel_guard), p.qb,
+                                     &live[L_QB], p.qb_cap, ctl, p.tn.chunk);
+                else
+                    warp_push_chunks<true>(large, v, d, p.qb, &live[L_QB], p.qb_cap, ctl, p.tn.chunk);
+            }
             walk_batch(p.ci, large ? -1 : v, rs, large ? 0 : (int)d, f);
         };
 
@@ -737,7 +848,16 @@ __device__ void run_async(const Params<Off> &p, GridDom &dom, unsigned *s_tmp,
         // small vertices, then (vertex, chunk) entries)
         const unsigned vb = batch_width(nfs, nfb, nwarps);
         unsigned long long walked = 0;   // listed entries walked, not yet added to `done`
-        {
+        if (resumed) {   // vertices of any degree
+            const unsigned w = batch_width(nfs, 0, nwarps);
+            for (unsigned unit = gwarp; unit * w < nfs; unit += nwarps) {
+                const unsigned idx = unit * w + lane;
+                int v = -1;
+                if (lane < w && idx < nfs) v = ldcg(p.fs + p.tail->lo + idx);
+                walk_vertices(v);
+                walked += min(w, nfs - unit * w);
+            }
+        } else {
             const unsigned nbatch = (nfs + vb - 1u) / vb;
             for (unsigned unit = gwarp; unit < nbatch + nfb; unit += nwarps) {
                 if (unit < nbatch) {
@@ -891,6 +1011,8 @@ __device__ void run_async(const Params<Off> &p, GridDom &dom, unsigned *s_tmp,
         clk.end(st, kPhLevel, nfs + nfb);
         k = k + 1;
     }
+    if (kTail && dom.leader()) p.tail->mode = kTailDone;
+    return true;
 }
 
 }  // namespace peel

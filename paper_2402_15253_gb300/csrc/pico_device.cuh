@@ -102,6 +102,7 @@ struct Ctrl {
     Line stat;                // w[0] status, w[1] CTAs that finished
     Line live;                // counters updated with atomics
     Line snap[2];             // live counters as of the last barrier (by parity)
+    Line tail;                // state shared by the launches of one PeelOne run (TailState)
     unsigned long long stats[kStCount];
 };
 
@@ -338,8 +339,9 @@ __device__ __forceinline__ void fold_block(Ctrl *c, unsigned long long *st)
 
 // Called once by every CTA at the end of a persistent kernel: folds the CTA's
 // statistics into the call's control block; the last CTA publishes the
-// status and statistics to the per-device LastResult.
-__device__ __forceinline__ void finish_block(Ctrl *c, LastResult *last, int algo,
+// status and statistics to the per-device LastResult. True for the thread that
+// published them.
+__device__ __forceinline__ bool finish_block(Ctrl *c, LastResult *last, int algo,
                                              const unsigned long long *local, int nlocal)
 {
     __syncthreads();
@@ -357,8 +359,10 @@ __device__ __forceinline__ void finish_block(Ctrl *c, LastResult *last, int algo
                 last->stats[i] = atomicAdd(&c->stats[i], 0ull);
             last->stats[kStBlocks] = gridDim.x;
             __threadfence();
+            return true;
         }
     }
+    return false;
 }
 
 // ---------------------------------------------------------------------------
@@ -440,53 +444,90 @@ __device__ __forceinline__ void block_min_to(int v, int *target, int *s)
 // ---------------------------------------------------------------------------
 // load-balanced adjacency expansion
 // ---------------------------------------------------------------------------
-// Writes reserved chunk entries: every lane with nch > 0 owns entries
-// pos .. pos + nch - 1 of vertex v (reserved by the caller). A lane writes a
-// short list itself; the warp writes the longer ones (hubs) together.
-__device__ __forceinline__ void warp_fill_chunks(unsigned nch, unsigned pos, int v, int2 *list)
+// Reserves n consecutive slots of *counter for every lane (all lanes call; one
+// atomic per warp, none when no lane asks). Returns the lane's first slot.
+__device__ __forceinline__ unsigned warp_reserve(unsigned *counter, unsigned n)
+{
+    const unsigned asking = __ballot_sync(kFull, n > 0);
+    if (asking == 0) return 0;
+    const unsigned lane = threadIdx.x & 31;
+    unsigned incl = n, base = 0;
+    if (asking & (asking - 1)) {
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned y = __shfl_up_sync(kFull, incl, o);
+            if ((int)lane >= o) incl += y;
+        }
+        if (lane == 31) base = atomicAdd(counter, incl);
+        return __shfl_sync(kFull, base, 31) + incl - n;
+    }
+    const int src = __ffs(asking) - 1;
+    if ((int)lane == src) base = atomicAdd(counter, n);
+    return __shfl_sync(kFull, base, src);
+}
+
+// Writes reserved entries: every lane with nch > 0 owns entries
+// pos .. pos + nch - 1 of list; entry(lane, c) is the c-th one of a lane's. A
+// lane writes a short list itself; the warp writes the longer ones (hubs)
+// together.
+template <bool kRelaxedStores, typename E>
+__device__ __forceinline__ void warp_fill(unsigned nch, unsigned pos, int2 *list, const E &entry)
 {
     constexpr unsigned kOwn = 8;
     const int lane = threadIdx.x & 31;
     if (nch <= kOwn)
-        for (unsigned c = 0; c < nch; ++c) list[pos + c] = make_int2(v, (int)c);
+        for (unsigned c = 0; c < nch; ++c) {
+            const int2 e = entry(lane, c);
+            if (kRelaxedStores) st_relaxed(list + pos + c, e);
+            else list[pos + c] = e;
+        }
     unsigned m = __ballot_sync(kFull, nch > kOwn);
     while (m) {
         const int src = __ffs(m) - 1;
         m &= m - 1;
         const unsigned nn = __shfl_sync(kFull, nch, src), pp = __shfl_sync(kFull, pos, src);
-        const int vv = __shfl_sync(kFull, v, src);
-        for (unsigned c = lane; c < nn; c += 32) list[pp + c] = make_int2(vv, (int)c);
+        entry.take(src);
+        for (unsigned c = lane; c < nn; c += 32) {
+            const int2 e = entry(-1, c);
+            if (kRelaxedStores) st_relaxed(list + pp + c, e);
+            else list[pp + c] = e;
+        }
     }
 }
 
+// (vertex, chunk) entries of the lane's vertex v.
+struct ChunkEntry {
+    int v;
+    mutable int other = 0;
+    __device__ __forceinline__ explicit ChunkEntry(int vertex) : v(vertex) {}
+    __device__ __forceinline__ void take(int src) const { other = __shfl_sync(kFull, v, src); }
+    __device__ __forceinline__ int2 operator()(int lane, unsigned c) const
+    {
+        return make_int2(lane >= 0 ? v : other, (int)c);
+    }
+};
+
+__device__ __forceinline__ void warp_fill_chunks(unsigned nch, unsigned pos, int v, int2 *list)
+{
+    warp_fill<false>(nch, pos, list, ChunkEntry(v));
+}
+
 // Warp-cooperative append of the chunk entries of large vertices: every
-// lane with `pred` owns vertex v of degree d; the whole warp writes the
-// ceil(d / chunk) entries of each such vertex in turn.
+// lane with `pred` owns vertex v of degree d and receives ceil(d / chunk)
+// entries. One counter update per warp: with one per vertex, a residual scan
+// that finds many of them waits for as many atomics in a row.
 template <bool kRelaxedStores = false>
 __device__ __forceinline__ void warp_push_chunks(bool pred, int v, long long d, int2 *list,
                                                  unsigned *counter, unsigned cap, Ctrl *ctl,
                                                  int chunk)
 {
-    const int lane = threadIdx.x & 31;
-    unsigned m = __ballot_sync(kFull, pred);
-    while (m) {
-        const int src = __ffs(m) - 1;
-        m &= m - 1;
-        const int vv = __shfl_sync(kFull, v, src);
-        const long long dd = __shfl_sync(kFull, d, src);
-        const unsigned nch = (unsigned)((dd + chunk - 1) / chunk);
-        unsigned pos = 0;
-        if (lane == 0) pos = atomicAdd(counter, nch);
-        pos = __shfl_sync(kFull, pos, 0);
-        if ((unsigned long long)pos + nch > cap) {
-            if (lane == 0) set_error(ctl, kErrNotConverged);
-            continue;
-        }
-        for (unsigned c = lane; c < nch; c += 32) {
-            if (kRelaxedStores) st_relaxed(list + pos + c, make_int2(vv, (int)c));
-            else list[pos + c] = make_int2(vv, (int)c);
-        }
+    unsigned nch = pred ? (unsigned)((d + chunk - 1) / chunk) : 0u;
+    const unsigned pos = warp_reserve(counter, nch);
+    if (nch > 0 && (unsigned long long)pos + nch > cap) {
+        set_error(ctl, kErrNotConverged);
+        nch = 0;
     }
+    if (__any_sync(kFull, nch > 0)) warp_fill<kRelaxedStores>(nch, pos, list, ChunkEntry(v));
 }
 
 // Default number of arcs a lane issues per step of expand(): their loads and

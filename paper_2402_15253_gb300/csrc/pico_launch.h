@@ -92,6 +92,28 @@ int launch_peelone(const Off *rp, const int *ci, long long n, long long m, int *
                    void *ws, LastResult *last, cudaStream_t stream, const LaunchCfg &cfg,
                    int mode = 0);
 
+namespace peel {
+template <typename Off>
+struct Params;
+struct TailState;
+}  // namespace peel
+
+// Whether a graph of this size is peeled in one CTA's shared memory
+// (launch_local) instead of by the grid kernel.
+bool peelone_local(long long n, long long m);
+
+// The shared-memory form; p: carved scratch with the control block zeroed.
+// tail: the launch does nothing when *tail says the call is published.
+template <typename Off>
+int launch_local(const peel::Params<Off> &p, long long m, const peel::TailState *tail,
+                 LastResult *last, cudaStream_t stream, const LaunchCfg &cfg);
+
+// The launches of the cluster kernel and the grid kernel that follow a first
+// launch of the grid kernel (peel::run_async with kTail), which left *p.tail.
+template <typename Off>
+int launch_turns(const peel::Params<Off> &p, long long m, LastResult *last, cudaStream_t stream,
+                 const LaunchCfg &cfg, int ctas);
+
 // init_est: start from these estimates (core maintenance; may alias core)
 template <typename Off>
 int launch_histocore(const Off *rp, const int *ci, long long n, long long m, int *core,
