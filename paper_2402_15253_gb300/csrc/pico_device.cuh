@@ -117,8 +117,10 @@ struct TraceEntry {
 // Per-device record of the most recent call, read by pico_get_stats,
 // pico_last_device_status and pico_get_trace.
 struct LastResult {
-    int status;               // sticky: first error since the last read
+    int status;               // sticky: first error since the last read ...
     int pad;
+    int *mapped;              // ... kept here, in host memory, instead (unless null): the host
+                              // then reads it without a copy
     long long algo;
     unsigned long long stats[kStCount];
     unsigned trace_len;
@@ -353,12 +355,15 @@ __device__ __forceinline__ bool finish_block(Ctrl *c, LastResult *last, int algo
         if (done == gridDim.x - 1) {
             __threadfence();
             int st = status_of(c);
-            if (st != 0) atomicCAS(&last->status, 0, st);
+            if (st != 0) {
+                if (last->mapped) atomicCAS_system(last->mapped, 0, st);
+                else atomicCAS(&last->status, 0, st);
+            }
             last->algo = algo;
             for (int i = 0; i < kStCount; ++i)
                 last->stats[i] = atomicAdd(&c->stats[i], 0ull);
             last->stats[kStBlocks] = gridDim.x;
-            __threadfence();
+            __threadfence_system();
             return true;
         }
     }
