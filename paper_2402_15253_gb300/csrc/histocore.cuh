@@ -65,6 +65,17 @@
 // with an acquire at GPU scope, after which a weak load observes every write
 // made before the barrier, so no line cached in an earlier phase is read.
 //
+// Compacted chunks. A pushed edit reaches u only when K = core[u] is above y,
+// and the neighbours of a hub mostly lie far below: on a Chung-Lu graph of 2^24
+// vertices a round that changes 2,000 hubs gathers 50 M records to edit 1 % of
+// them, at the rate L2 serves them. So the first push of a chunk writes the
+// neighbours with K > y / 2 to the chunk's place in an array like col_idx
+// (`near`: their number, the bound y / 2, the neighbours). Estimates only fall,
+// so while y stays at or above the bound the others cannot be above y either,
+// and later pushes walk that list; below the bound it is built again. A chunk
+// most of whose neighbours qualify is left alone. Replayed on R-MAT scale 18 and
+// Chung-Lu 2^18, half and an eighth of the pushed arcs remain.
+//
 // Load balance. V_cnt is kept as three lists by the estimate K that SumHisto
 // will walk down from: K <= 32 one thread per vertex, K <= 2048 one warp per
 // vertex (32 slots per step, warp suffix scan), larger K one CTA per vertex.
@@ -136,7 +147,13 @@ struct Params {
     // rounded up to 4; zero between rounds); nullptr: pull rounds decide the
     // append at the edit, as push rounds do.
     unsigned char *cand = nullptr;
+    // Compacted chunks (m ints; nullptr: pushes walk every arc). The chunk that
+    // starts at arc s, if it has at least kNearMin arcs: near[s] is the number
+    // of neighbours listed from near[s + 2] on, or kNearNone (not built) or
+    // kNearFull (not worth it); near[s + 1] the bound.
+    int *near = nullptr;
 };
+constexpr int kNearMin = 16, kNearNone = -1, kNearFull = -2;
 
 // Packed {old, new} record: old << 16 | new when old <= 65534 (new < old);
 // kMvpWide otherwise (never a packed value, since new < old).
@@ -226,7 +243,10 @@ struct UpdateArc {
     unsigned *live_base;   // counters of the domain
     int par;               // parity of the next round's lists
     unsigned cap;          // slots of each list (n)
-    unsigned long long n_arcs = 0, n_atomics = 0;
+    int *list = nullptr;   // the walk lists the neighbours above `bound` here (warp-uniform)
+    int bound = 0;
+    int room = 0, listed = 0;
+    unsigned long long n_atomics = 0;
 
     __device__ __forceinline__ bool item(int v, int &x, int &y)
     {
@@ -248,18 +268,82 @@ struct UpdateArc {
             K[j] = (int)r.x;
             ru[j] = (Off)r.y;
         }
+        if (list) {   // invalid lanes hold K = 0
+            const unsigned lane = threadIdx.x & 31;
+#pragma unroll
+            for (int j = 0; j < kArcs; ++j) {
+                const unsigned b = __ballot_sync(kFull, K[j] > bound);
+                const int at = listed + __popc(b & ((1u << lane) - 1u));
+                if (K[j] > bound && at < room) list[at] = u[j];
+                listed += __popc(b);
+            }
+        }
         bool push[kArcs];
 #pragma unroll
         for (int j = 0; j < kArcs; ++j) {
-            push[j] = false;
-            if (valid[j]) {
-                ++n_arcs;
-                push[j] = edit_row(histo, ru[j], K[j], x[j], y[j], n_atomics);
-            }
+            push[j] = valid[j] && edit_row(histo, ru[j], K[j], x[j], y[j], n_atomics);
         }
         append_vcnt(push, u, K, live_base + 3 * par, tl, wl, bl, cap, ctl);
     }
 };
+
+// One warp pushes chunk c of changed vertex v, from its compacted list when
+// there is one for the vertex's new estimate (see Params::near).
+template <typename Off>
+__device__ __forceinline__ void push_chunk(const Params<Off> &p, int v, int c, UpdateArc<Off> &f)
+{
+    constexpr int U = UpdateArc<Off>::kArcs;
+    const int lane = threadIdx.x & 31;
+    const Off rs = p.rp[v], re = p.rp[v + 1];
+    const Off s = rs + (Off)c * p.tn.chunk;
+    int len = (int)(re - s < (Off)p.tn.chunk ? re - s : (Off)p.tn.chunk);
+    int x = 0, y = 0;
+    f.item(v, x, y);
+    const int *arcs = p.ci + s;
+    bool build = false, compacted = false;
+    if (p.near && len >= kNearMin) {
+        int *head = p.near + s;
+        const int h = ldcg(head + (lane & 1));   // lane 0: the number, lane 1: the bound
+        const int number = __shfl_sync(kFull, h, 0), bound = __shfl_sync(kFull, h, 1);
+        if (number != kNearNone && y >= bound) {
+            if (number >= 0) {
+                arcs = head + 2;
+                len = number;
+                compacted = true;
+            }
+        } else {
+            build = true;
+            f.list = head + 2;
+            f.bound = y >> 1;
+            f.room = len - len / 4 - 2;   // the list and its head fit the chunk
+            f.listed = 0;
+        }
+    }
+    for (int e0 = 0; e0 < len; e0 += 32 * U) {
+        bool valid[U];
+        int vo[U], u[U], xo[U], yo[U];
+        Off rso[U];
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+            const int e = e0 + 32 * j + lane;
+            valid[j] = e < len;
+            // a list may have been written in this launch, by another CTA
+            u[j] = valid[j] ? (compacted ? ldcg(arcs + e) : __ldg(arcs + e)) : -1;
+            vo[j] = v;
+            rso[j] = rs;
+            xo[j] = x;
+            yo[j] = y;
+        }
+        f.arcs(valid, vo, u, rso, xo, yo);
+    }
+    if (build) {
+        if (lane == 0) {
+            p.near[s] = f.listed <= f.room ? f.listed : kNearFull;
+            p.near[s + 1] = f.bound;
+        }
+        f.list = nullptr;
+    }
+}
 
 // Pull form of UpdateHisto: arcs of every vertex u whose estimate K is above
 // the smallest new estimate of the round; the edit of arc (u, w) is the one
@@ -640,6 +724,11 @@ __device__ void run(const Params<Off> &p0, Dom &dom, unsigned *s_tmp, unsigned l
     // InitHisto
     {
         InitArc<Off> f{p.vinfo, p.histo};
+        if (p.near)   // no chunk is compacted yet
+            for (unsigned i = tid; i < nib; i += nthreads) {
+                const int2 e = __ldcg(ilist + i);
+                p.near[p.rp[e.x] + (Off)e.y * p.tn.chunk] = kNearNone;
+            }
         expand(p.rp, p.ci, (const int *)nullptr, (unsigned)n, ilist, nib, gwarp, nwarps, f, p.tn);
         arcs += f.n_arcs;
         atomics += f.n_arcs;
@@ -762,9 +851,19 @@ __device__ void run(const Params<Off> &p0, Dom &dom, unsigned *s_tmp, unsigned l
         } else {
             UpdateArc<Off> f{p.vinfo, p.mv[par], p.histo, p.tl[np], p.wl[np], p.bl[np],
                              ctl,     live,      np,      (unsigned)n};
-            expand(p.rp, p.ci, p.us, nus, p.ub, nub, gwarp, nwarps, f, p.tn,
-                   batch_width(nus, nub, nwarps));
-            arcs += f.n_arcs;
+            const unsigned vb = batch_width(nus, nub, nwarps), nbatch = (nus + vb - 1u) / vb;
+            const unsigned lane = threadIdx.x & 31;
+            for (unsigned unit = gwarp; unit < nbatch + nub; unit += nwarps) {
+                if (unit < nbatch) {
+                    const unsigned idx = unit * vb + lane;
+                    const int v = lane < vb && idx < nus ? ldcg(p.us + idx) : -1;
+                    walk_small_batch(p.rp, p.ci, v, f, p.tn.small_deg);
+                } else {
+                    const int2 ent = __ldcg(p.ub + (unit - nbatch));   // written by other CTAs
+                    push_chunk(p, ent.x, ent.y, f);
+                }
+            }
+            arcs += acc.arcs;   // the changed vertices' arcs, as Alg. 6 scans them
             atomics += f.n_atomics;
         }
         if (!dom.sync()) return;
