@@ -13,12 +13,14 @@
 //          are as many of them as of the others, every arc has its reverse.
 //   arcs   (only when the quick pass found something) every arc's defects, each
 //          reverse looked up.
-// The quick pass shares the arcs out evenly, 512 to a warp: one warp per row
+// The quick pass shares the arcs out evenly, up to 512 to a warp: one warp per row
 // leaves a hub's row to a single warp (R-MAT scale 20, n 1.0 M, m 31 M: 9.2 ms).
 // What remains is its gathers: two row bounds per arc, and a lookup in the
 // shorter row for half of them. Each kernel ORs what it finds into one device
 // word. Every load is bounds-checked first, so a malformed graph becomes a
 // reported defect, never an out-of-range access.
+#include <algorithm>
+
 #include "pico.h"
 #include "pico_device.cuh"
 #include "pico_launch.h"
@@ -44,23 +46,25 @@ __global__ void __launch_bounds__(256)
     if (bad) atomicOr(flag, PICO_DEFECT_ROWS);
 }
 
-constexpr int kSegment = 512;   // arcs of a warp's turn in the quick pass
+constexpr int kSegment = 512;   // most arcs of a warp's turn in the quick pass
 
+// segment: arcs of a warp's turn, a multiple of 32
 template <typename Off>
 __global__ void __launch_bounds__(256)
-    validate_quick(const Off *rp, const int *ci, long long n, long long m, ValidateWords *words)
+    validate_quick(const Off *rp, const int *ci, long long n, long long m, int segment,
+                   ValidateWords *words)
 {
     __shared__ long long s_sum[8];
     // the rows kernel ran before on this stream: its word is final here
     if (ld_relaxed(&words->defects) & PICO_DEFECT_ROWS) return;
     const int lane = threadIdx.x & 31;
     const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
-    const long long nseg = (m + kSegment - 1) / kSegment;
+    const long long nseg = (m + segment - 1) / segment;
     bool bad = false;
     int excess = 0;   // arcs looked up minus the others
     for (long long seg = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; seg < nseg;
          seg += nw) {
-        const long long a0 = seg * kSegment, a1 = a0 + kSegment < m ? a0 + kSegment : m;
+        const long long a0 = seg * segment, a1 = a0 + segment < m ? a0 + segment : m;
         // the last row that starts at or before a0, by 32-way search: rp[lo] <= a0 < rp[hi]
         long long lo = 0, hi = n;
         while (hi - lo > 1) {
@@ -169,10 +173,17 @@ template <typename Off>
 int launch_validate(const Off *rp, const int *ci, long long n, long long m, ValidateWords *words,
                     cudaStream_t stream, const LaunchCfg &cfg)
 {
-    const unsigned blocks = (unsigned)(cfg.sms > 0 ? cfg.sms * 8 : 1024);
+    // no more CTAs than the vertices, or the shares of arcs, occupy: on a small
+    // graph most of a launch's time is setting up CTAs; and shares so small
+    // that every warp has one: a share is walked 32 arcs at a time
+    const long long most = cfg.sms > 0 ? cfg.sms * 8 : 1024;
+    const int segment =
+        (int)std::min<long long>(kSegment, std::max<long long>(32, (m / (8 * most) + 31) & ~31ll));
+    const unsigned blocks = (unsigned)std::min<long long>(most, n / 256 + 1);
+    const unsigned shares = (unsigned)std::min<long long>(most, m / (8 * segment) + 1);
     validate_rows<Off><<<blocks, 256, 0, stream>>>(rp, n, m, &words->defects);
     if (cudaGetLastError() != cudaSuccess) return -3;
-    validate_quick<Off><<<blocks, 256, 0, stream>>>(rp, ci, n, m, words);
+    validate_quick<Off><<<shares, 256, 0, stream>>>(rp, ci, n, m, segment, words);
     if (cudaGetLastError() != cudaSuccess) return -3;
     validate_arcs<Off><<<blocks, 256, 0, stream>>>(rp, ci, n, words);
     if (cudaGetLastError() != cudaSuccess) return -3;
