@@ -43,6 +43,8 @@ constexpr int kPeelCtas = 4;                    // PeelOne: CTAs per cluster
 constexpr int kWideThreads = 1024;              // PeelOne: threads per CTA of large and middle graphs
 constexpr int kTinyThreads = 128;               // ... and of tiny ones
 constexpr int kTinyVertices = 2048;
+constexpr size_t kTinySmem = 26 * 1024;         // eight CTAs share an SM's 228 KB
+static_assert(kTinySmem >= 16 * kTinyVertices / 2 + 4096, "row offsets of a tiny graph must fit");
 
 // control words of the batched launch (in Ctrl::live): tickets of the classes,
 // the number of graphs in the first class, and in the first two
@@ -271,7 +273,11 @@ __global__ void __launch_bounds__(kWideThreads, 1) batched_peel_kernel(BatchPara
         __syncthreads();
         if (t >= nmiddle || status_of(bp.ctl) != 0) break;
         const peel::LocalParams<int> p = local_params(bp, bp.order[t]);
-        const peel::LocalStats s = peel::run_local<int, peel::LocalWide, false>(p, smem, 0, 1);
+        const bool rows = peel::local_smem_bytes<peel::LocalWide>(p.n, peel::kKeepRows) <=
+                          peel::kLocalSmem;
+        const peel::LocalStats s =
+            rows ? peel::run_local<int, peel::LocalWide, false, peel::kKeepRows>(p, smem, 0, 1)
+                 : peel::run_local<int, peel::LocalWide, false>(p, smem, 0, 1);
         if (threadIdx.x == 0) peel::add_stats(st, s, p.n, p.m);
         __syncthreads();
     }
@@ -300,7 +306,11 @@ __global__ void __launch_bounds__(kTinyThreads, 8) batched_tiny_kernel(BatchPara
         if (t >= bp.G || status_of(bp.ctl) != 0) break;
         const peel::LocalParams<int> p = local_params(bp, bp.order[t]);
         if (p.n <= 0) continue;
-        const peel::LocalStats s = peel::run_local<int, peel::LocalTiny, false>(p, smem, 0, 1);
+        const bool whole = peel::local_smem_bytes<peel::LocalTiny>(p.n, peel::kKeepGraph, p.m) <=
+                           kTinySmem;
+        const peel::LocalStats s =
+            whole ? peel::run_local<int, peel::LocalTiny, false, peel::kKeepGraph>(p, smem, 0, 1)
+                  : peel::run_local<int, peel::LocalTiny, false, peel::kKeepRows>(p, smem, 0, 1);
         if (threadIdx.x == 0) peel::add_stats(st, s, p.n, p.m);
         __syncthreads();
     }
@@ -404,11 +414,11 @@ int launch_batched(const int64_t *vtx_off, const int64_t *arc_off, int G, const 
         const long long wide = std::min<long long>(G, total_n / (kTinyVertices + 1));
         if (wide > 0 &&
             launch_clusters((const void *)batched_peel_kernel, kPeelCtas, kWideThreads,
-                            peel::local_smem_bytes<peel::LocalWide>(peel::kLocalSlots), cfg.sms,
+                            peel::kLocalSmem, cfg.sms,
                             wide, occ_wide[dev], args, stream) != cudaSuccess)
             return -3;
         if (launch_clusters((const void *)batched_tiny_kernel, 1, kTinyThreads,
-                            peel::local_smem_bytes<peel::LocalTiny>(kTinyVertices), cfg.sms * 8, G,
+                            kTinySmem, cfg.sms * 8, G,
                             occ_tiny[dev], args, stream) != cudaSuccess)
             return -3;
         return 0;

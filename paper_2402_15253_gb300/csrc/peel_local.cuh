@@ -13,10 +13,10 @@
 //   one CTA    (n <= kLocalSlots) owns every vertex.
 //   a cluster  of c CTAs (n <= c * kLocalSlots): CTA r owns the vertices
 //              [r * per, (r + 1) * per). Every CTA walks every frontier arc
-//              and applies the ones that end at its own vertices. Remote
-//              atomics would let the CTAs share the walk, but distributed
-//              shared memory serves 0.32 of them per clock and SM (measured),
-//              less than one SM's own shared memory does in a cluster of 16.
+//              and applies the ones that end at its own vertices. Sharing the
+//              walk and decrementing through distributed shared memory (0.37
+//              atomics per clock and SM, measured) takes the same time: 184
+//              graphs of 51,201 to 200,000 vertices 11.3 ms either way.
 //
 // Queue: each CTA queues its own vertices (each once over the run) in its
 // part of a global array, level by level; a single CTA keeps the first
@@ -45,7 +45,7 @@ constexpr int kLocalSlots = 51200;   // residual degrees per CTA (200 KB of shar
 // Rows longer than a piece are split over the CTA's warps: into 128 arcs (one
 // step of a warp) when a wave has no more rows than warps, else 256.
 __device__ __forceinline__ int local_piece(unsigned vb) { return vb == 1u ? 128 : 256; }
-constexpr int kLocalMaxCtas = 8;
+constexpr int kLocalMaxCtas = 4;
 
 // Capacities of a CTA's shared lists: queue entries of a level kept in shared
 // memory, and chunk entries listed at once.
@@ -86,12 +86,33 @@ struct LocalStats {
     int kmax = 0;
 };
 
-// Dynamic shared memory of a CTA that owns up to `slots` vertices.
+// What a CTA that peels a graph alone keeps of it in shared memory besides the
+// residual degrees: the row offsets, or all of it. A wave of a small graph is a
+// chain of dependent accesses (row bounds, columns, decrements), and each of
+// the first two takes some 500 clocks from L2 and 30 from shared memory.
+enum : int { kKeepNone = 0, kKeepRows = 1, kKeepGraph = 2 };
+
+// Dynamic shared memory of a CTA that owns `n` vertices (and the m arcs of the
+// whole graph, if kept).
 template <typename Cap>
-__host__ __device__ inline size_t local_smem_bytes(int slots)
+__host__ __device__ inline size_t local_smem_bytes(long long n, int kept = kKeepNone, long long m = 0)
 {
-    return ((sizeof(LocalShared<Cap>) + 15) & ~size_t(15)) + (size_t)((slots + 3) & ~3) * sizeof(int);
+    const size_t slots = (size_t)((n + 3) & ~3ll);
+    size_t b = ((sizeof(LocalShared<Cap>) + 15) & ~size_t(15)) + slots * sizeof(int);
+    if (kept != kKeepNone) b += (slots + 4) * sizeof(int);
+    if (kept == kKeepGraph) b += (size_t)m * sizeof(int);
+    return b;
 }
+
+// The most that fits `bytes` of dynamic shared memory.
+template <typename Cap>
+__host__ __device__ inline int local_kept(long long n, long long m, size_t bytes)
+{
+    if (local_smem_bytes<Cap>(n, kKeepGraph, m) <= bytes) return kKeepGraph;
+    return local_smem_bytes<Cap>(n, kKeepRows) <= bytes ? kKeepRows : kKeepNone;
+}
+
+constexpr size_t kLocalSmem = 227 * 1024 - 2048;   // dynamic shared memory of a wide CTA
 
 __device__ __forceinline__ unsigned shared_addr(const void *p)
 {
@@ -120,13 +141,12 @@ __device__ __forceinline__ int shared_dec(unsigned addr)
 // lanes with d > 0 come first). A 32-arc window's owners follow from the
 // rows that start in it: one warp-wide OR and a population count, where a
 // search over the row starts would take five dependent shuffles. f takes
-// kLocalU windows at a time: f.arcs(valid, u), called by all 32 lanes.
-constexpr int kLocalU = 4;
-
-template <typename Off, typename F>
+// F::kArcs windows at a time: f.arcs(valid, u), called by all 32 lanes.
+// kShared: ci is in shared memory.
+template <bool kShared, typename Off, typename F>
 __device__ __forceinline__ void walk_rows(const int *__restrict__ ci, Off rs, int d, F &f)
 {
-    constexpr int U = kLocalU;
+    constexpr int U = F::kArcs;
     const int lane = threadIdx.x & 31;
     int incl = d;
 #pragma unroll
@@ -153,7 +173,7 @@ __device__ __forceinline__ void walk_rows(const int *__restrict__ ci, Off rs, in
                 const int owner = before + __popc(starts & (0xffffffffu >> (31 - lane)));
                 before += __popc(starts);
                 const Off o = __shfl_sync(kFull, off, owner & 31);
-                if (valid[j]) u[j] = __ldg(ci + o + e);
+                if (valid[j]) u[j] = kShared ? ci[o + e] : __ldg(ci + o + e);
             }
         }
         f.arcs(valid, u);
@@ -161,10 +181,10 @@ __device__ __forceinline__ void walk_rows(const int *__restrict__ ci, Off rs, in
 }
 
 // One warp walks `len` consecutive arcs.
-template <typename F>
+template <bool kShared, typename F>
 __device__ __forceinline__ void walk_arcs(const int *__restrict__ c, int len, F &f)
 {
-    constexpr int U = kLocalU;
+    constexpr int U = F::kArcs;
     const int lane = threadIdx.x & 31;
     for (int base = 0; base < len; base += 32 * U) {
         bool valid[U];
@@ -173,7 +193,7 @@ __device__ __forceinline__ void walk_arcs(const int *__restrict__ c, int len, F 
         for (int j = 0; j < U; ++j) {
             const int e = base + 32 * j + lane;
             valid[j] = e < len;
-            u[j] = valid[j] ? __ldg(c + e) : -1;
+            u[j] = valid[j] ? (kShared ? c[e] : __ldg(c + e)) : -1;
         }
         f.arcs(valid, u);
     }
@@ -196,12 +216,17 @@ __device__ __forceinline__ void pack_rows(Off &rs, int &d)
     d = lane < (unsigned)__popc(have) ? d2 : 0;
 }
 
-template <typename Off, typename Cap, bool kCluster>
+template <typename Off, typename Cap, bool kCluster, int kKept>
 struct LocalPeel {
+    // a whole graph in shared memory is small: its waves go through this code
+    // once, and fetching the instructions is part of their latency
+    static constexpr int kArcs = kKept == kKeepGraph ? 2 : 4;
+    static constexpr bool kCols = kKept == kKeepGraph;
     const LocalParams<Off> &p;
     LocalShared<Cap> &sh;
     int *res;
     unsigned res_addr;     // its shared-memory address
+    int *rows, *cols;      // copies of row_ptr and col_idx, if kept
     unsigned rank, ctas;   // this CTA in its cluster
     int per;               // vertices per CTA
     int vbase, cnt;        // own vertices
@@ -244,18 +269,46 @@ struct LocalPeel {
 
     // The decrements of a step's arcs (walk_rows, walk_arcs): all issued
     // before the first result is used.
-    __device__ __forceinline__ void arcs(const bool (&valid)[kLocalU], const int (&u)[kLocalU])
+    __device__ __forceinline__ void arcs(const bool (&valid)[kArcs], const int (&u)[kArcs])
     {
-        int old[kLocalU];
+        int old[kArcs];
 #pragma unroll
-        for (int j = 0; j < kLocalU; ++j) {
+        for (int j = 0; j < kArcs; ++j) {
             const unsigned x = (unsigned)(u[j] - vbase);
             old[j] = valid[j] && x < (unsigned)cnt ? shared_dec(res_addr + 4u * x) : 0;
         }
-        bool push[kLocalU];
+        bool push[kArcs];
 #pragma unroll
-        for (int j = 0; j < kLocalU; ++j) push[j] = old[j] == k + 1;   // k + 1 > 0
+        for (int j = 0; j < kArcs; ++j) {
+            push[j] = old[j] == k + 1;   // k + 1 > 0
+        }
         queue_own(push, u);
+    }
+
+    // Queues the own vertices whose residual degree is k, and records the
+    // smallest one above k.
+    __device__ __forceinline__ void collect()
+    {
+        const int tid = (int)threadIdx.x, T = (int)blockDim.x;
+        int mn = INT_MAX;
+        const int4 *r4 = reinterpret_cast<const int4 *>(res);
+        for (int base = 0; base < cnt; base += 4 * T) {
+            const int i = base + 4 * tid;
+            int4 c = make_int4(0, 0, 0, 0);
+            if (i < cnt) c = r4[i >> 2];   // the padding holds 0 < k
+            const int cv[4] = {c.x, c.y, c.z, c.w};
+            bool push[4];
+            int v[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                push[j] = cv[j] == k;
+                if (cv[j] > k) mn = min(mn, cv[j]);
+                v[j] = vbase + i + j;
+            }
+            queue_own(push, v);
+        }
+        mn = __reduce_min_sync(kFull, mn);
+        if ((tid & 31) == 0 && mn != INT_MAX) atomicMin(&sh.vmin[ph], mn);
     }
 
     // Ends a phase: every CTA learns every CTA's count (and, after a scan, its
@@ -301,6 +354,19 @@ struct LocalPeel {
         return t;
     }
 
+    __device__ __forceinline__ void row(int v, Off &rs, int &d) const
+    {
+        if (kKept != kKeepNone) {
+            const int a = rows[v];
+            rs = (Off)a;
+            d = rows[v + 1] - a;
+        } else {
+            rs = p.rp[v];
+            d = (int)(p.rp[v + 1] - rs);
+        }
+    }
+    __device__ __forceinline__ const int *columns() const { return kCols ? cols : p.ci; }
+
     // Walks the vertices queued in phase slot `s`; q[r] is the level's queue
     // position of CTA r's first one.
     __device__ __forceinline__ void wave(unsigned s, unsigned total, const int (&q)[kLocalMaxCtas])
@@ -330,10 +396,7 @@ struct LocalPeel {
             }
             Off rs = 0;
             int d = 0;
-            if (v >= 0) {
-                rs = p.rp[v];
-                d = (int)(p.rp[v + 1] - rs);
-            }
+            if (v >= 0) row(v, rs, d);
             unsigned bigs = __ballot_sync(kFull, d > piece);
             while (bigs) {   // list the chunks of long rows, or walk them here when the list is full
                 const int src = __ffs(bigs) - 1;
@@ -350,19 +413,20 @@ struct LocalPeel {
                     sh.c_start[pos + c] = (unsigned long long)(s0 + (Off)c * size);
                     sh.c_len[pos + c] = fits ? min(size, dd - (int)c * size) : 0;
                 }
-                if (!fits) walk_arcs(p.ci + s0, dd, *this);
+                if (!fits) walk_arcs<kCols>(columns() + s0, dd, *this);
             }
             if (d > piece) d = 0;
             if (vb == 1u) {
-                walk_arcs(p.ci + __shfl_sync(kFull, rs, 0), __shfl_sync(kFull, d, 0), *this);
+                walk_arcs<kCols>(columns() + __shfl_sync(kFull, rs, 0), __shfl_sync(kFull, d, 0), *this);
             } else {
                 pack_rows(rs, d);
-                walk_rows(p.ci, rs, d, *this);
+                walk_rows<kCols>(columns(), rs, d, *this);
             }
         }
         __syncthreads();
         const unsigned nch = min(sh.nchunk[ph], (unsigned)Cap::kChunks);
-        for (unsigned c = warp; c < nch; c += nw) walk_arcs(p.ci + sh.c_start[c], sh.c_len[c], *this);
+        for (unsigned c = warp; c < nch; c += nw)
+            walk_arcs<kCols>(columns() + sh.c_start[c], sh.c_len[c], *this);
     }
 
     // Peels the graph. Every thread of the CTA (cluster) calls it.
@@ -384,14 +448,23 @@ struct LocalPeel {
             int d = 0;
             if (i < cnt) {
                 const int v = vbase + i;
-                d = (int)(p.rp[v + 1] - p.rp[v]);
+                const Off rs = p.rp[v];
+                d = (int)(p.rp[v + 1] - rs);
                 if (d == 0) p.core[v] = 0;
+                if (kKept != kKeepNone) {
+                    rows[v] = (int)rs;
+                    if (v + 1 == cnt) rows[v + 1] = (int)rs + d;
+                }
             }
             res[i] = d;
             if (d > 0) {
                 mn = min(mn, d);
                 ++linked;
             }
+        }
+        if (kCols) {
+#pragma unroll 8
+            for (int i = tid; i < (int)p.m; i += T) cols[i] = __ldg(p.ci + i);
         }
         linked = __reduce_add_sync(kFull, linked);
         if (lane == 0 && linked) atomicAdd(&sh.pushed[ph], linked);
@@ -410,25 +483,7 @@ struct LocalPeel {
             // scan: own vertices at k are the level's static frontier
             q0 = 0;
             ++st.scans;
-            mn = INT_MAX;
-            const int4 *r4 = reinterpret_cast<const int4 *>(res);
-            for (int base = 0; base < cnt; base += 4 * T) {
-                const int i = base + 4 * tid;
-                int4 c = make_int4(0, 0, 0, 0);
-                if (i < cnt) c = r4[i >> 2];
-                const int cv[4] = {c.x, c.y, c.z, c.w};
-                bool push[4];
-                int v[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    if (cv[j] > k) mn = min(mn, cv[j]);
-                    push[j] = cv[j] == k;   // padding holds 0 < k
-                    v[j] = vbase + i + j;
-                }
-                queue_own(push, v);
-            }
-            mn = __reduce_min_sync(kFull, mn);
-            if (lane == 0 && mn != INT_MAX) atomicMin(&sh.vmin[ph], mn);
+            collect();
             end_phase<true>();
             prev = ph == 0 ? 2 : ph - 1;
             unsigned total = total_of(prev);
@@ -471,14 +526,16 @@ struct LocalPeel {
     }
 };
 
-// smem: local_smem_bytes<Cap>(p.n / ctas rounded up) bytes of dynamic shared memory.
-template <typename Off, typename Cap, bool kCluster>
+// smem: local_smem_bytes<Cap>(...) bytes of dynamic shared memory.
+template <typename Off, typename Cap, bool kCluster, int kKept = kKeepNone>
 __device__ __forceinline__ LocalStats run_local(const LocalParams<Off> &p, char *smem, unsigned rank,
                                                 unsigned ctas)
 {
     LocalShared<Cap> &sh = *reinterpret_cast<LocalShared<Cap> *>(smem);
     int *res = reinterpret_cast<int *>(smem + ((sizeof(LocalShared<Cap>) + 15) & ~size_t(15)));
-    LocalPeel<Off, Cap, kCluster> lp{p, sh, res, shared_addr(res), rank, ctas};
+    int *rows = res + ((p.n + 3) & ~3);
+    LocalPeel<Off, Cap, kCluster, kKept> lp{p, sh, res, shared_addr(res), rows,
+                                            rows + ((p.n + 3) & ~3) + 4, rank, ctas};
     lp.per = kCluster ? (int)(((p.n + (int)ctas - 1) / (int)ctas + 3) & ~3) : p.n;
     lp.vbase = (int)rank * lp.per;
     lp.cnt = max(0, min(lp.per, p.n - lp.vbase));

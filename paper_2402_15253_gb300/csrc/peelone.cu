@@ -13,11 +13,11 @@
 namespace pico {
 namespace {
 
-// The shared-memory form: threads of its CTA, and half as many for the
-// smallest graphs, whose waves are a few rows and whose CTA barriers are
-// then cheaper (R-MAT scale 10: 137 against 144 us).
+// The shared-memory form: threads of its CTA, and half as many for graphs that
+// are kept there whole, whose waves are a few rows: idle warps take issue slots
+// and the CTA barrier is cheaper (R-MAT scale 10: 124 us with 512, 135 with
+// 1,024 threads; a path of 5,000 vertices: 2.34 and 2.67 ms).
 constexpr int kLocalThreads = 1024;
-constexpr long long kLocalNarrow = 2048;
 // One SM walks about 1.5 arcs per clock, so it loses to the grid where there
 // are many arcs and few levels (Erdos-Renyi, n 50,001, m 0.8 M, 9 levels: 504
 // against 266 us) and wins on skewed graphs up to this size (R-MAT scale 14, m
@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(peel::kTailThreads, 1)
 // A graph whose residual degrees fit the shared memory of one CTA
 // (peel_local.cuh). tail: another launch may have solved it already (nullptr:
 // none has).
-template <typename Off>
+template <typename Off, int kKept>
 __global__ void __launch_bounds__(kLocalThreads, 1)
     peelone_local_kernel(peel::LocalParams<Off> p, const peel::TailState *tail, LastResult *last)
 {
@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(kLocalThreads, 1)
     }
     __syncthreads();
     clk.start();
-    const peel::LocalStats s = peel::run_local<Off, peel::LocalWide, false>(p, smem, 0, 1);
+    const peel::LocalStats s = peel::run_local<Off, peel::LocalWide, false, kKept>(p, smem, 0, 1);
     if (threadIdx.x == 0) peel::add_stats(st, s, p.n, p.m);
     clk.end(st, kPhWaveMid, (unsigned)s.waves);
     finish_block(p.ctl, last, PICO_ALGO_PEELONE, st, kStCount);
@@ -240,16 +240,18 @@ template <typename Off>
 int launch_local(const peel::Params<Off> &p, long long m, const peel::TailState *tail,
                  LastResult *last, cudaStream_t stream, const LaunchCfg &cfg)
 {
-    static bool ready[64] = {};
-    const void *fn = (const void *)peelone_local_kernel<Off>;
-    if (!prepare_kernel(fn, peel::local_smem_bytes<peel::LocalWide>(peel::kLocalSlots), false,
-                        ready[cfg.device & 63]))
-        return -3;
+    static bool ready[3][64] = {};
+    const void *fns[3] = {(const void *)peelone_local_kernel<Off, peel::kKeepNone>,
+                          (const void *)peelone_local_kernel<Off, peel::kKeepRows>,
+                          (const void *)peelone_local_kernel<Off, peel::kKeepGraph>};
+    const int kept = peel::local_kept<peel::LocalWide>(p.n, m, peel::kLocalSmem);
+    const void *fn = fns[kept];
+    if (!prepare_kernel(fn, peel::kLocalSmem, false, ready[kept][cfg.device & 63])) return -3;
     peel::LocalParams<Off> lp{p.rp, p.ci, (int)p.n, m, p.core, p.qs, p.ctl};
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(1);
-    lc.blockDim = dim3(p.n <= kLocalNarrow ? kLocalThreads / 2 : kLocalThreads);
-    lc.dynamicSmemBytes = peel::local_smem_bytes<peel::LocalWide>((int)p.n);
+    lc.blockDim = dim3(kept == peel::kKeepGraph ? kLocalThreads / 2 : kLocalThreads);
+    lc.dynamicSmemBytes = peel::local_smem_bytes<peel::LocalWide>(p.n, kept, m);
     lc.stream = stream;
     void *args[] = {&lp, &tail, &last};
     return cudaLaunchKernelExC(&lc, fn, args) == cudaSuccess ? 0 : -3;
