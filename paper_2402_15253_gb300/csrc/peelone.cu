@@ -13,6 +13,10 @@
 namespace pico {
 namespace {
 
+// Percent of an SM's shared memory for the kernels that alternate: the same for
+// both, so that the SMs are not set up anew between them.
+constexpr int kTailCarveout = 50;
+
 // The shared-memory form: threads of its CTA, and half as many for graphs that
 // are kept there whole, whose waves are a few rows: idle warps take issue slots
 // and the CTA barrier is cheaper (R-MAT scale 10: 124 us with 512, 135 with
@@ -158,6 +162,10 @@ cudaError_t launch_tail(peel::Params<Off> &p, long long m, LastResult *last, cud
     static bool ready[64] = {};
     const void *fn = (const void *)peelone_tail_kernel<Off>;
     constexpr size_t smem = sizeof(peel::TailShared);
+    if (!ready[device & 63] &&
+        cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, kTailCarveout) !=
+            cudaSuccess)
+        return cudaErrorInvalidValue;
     if (!prepare_kernel(fn, smem, true, ready[device & 63])) return cudaErrorInvalidValue;
     cudaLaunchConfig_t lc = {};
     cudaLaunchAttribute attr[1];
@@ -176,12 +184,13 @@ cudaError_t launch_tail(peel::Params<Off> &p, long long m, LastResult *last, cud
 }
 
 // Launches that follow the grid kernel's first: cluster and grid kernel in turn.
-// A launch with nothing to do takes 4 to 5 us, so small graphs get few and end
-// with the cluster kernel (which walks 5 M arcs at worst in 0.4 ms); large ones
-// end with the grid kernel.
+// One with nothing to do takes 3.3 us, so small graphs get few and end with the
+// cluster kernel (which walks 5 M arcs at worst in 0.4 ms); large ones end with
+// the grid kernel. R-MAT scales 20 and 21 take 4.75 and 6.20 ms with six, 5.95
+// and 7.22 ms with four.
 int tail_launches(long long m)
 {
-    return m < (6 << 20) ? 1 : m < (12 << 20) ? 3 : m < (20 << 20) ? 4 : m < (32 << 20) ? 6 : 12;
+    return m < (6 << 20) ? 1 : m < (20 << 20) ? 3 : m < (120 << 20) ? 6 : 12;
 }
 
 // Reads a range (16 bytes a thread per step); the values are not used.
@@ -312,6 +321,10 @@ int launch_peelone(const Off *rp, const int *ci, long long n, long long m, int *
     }
     int &o = occ[async][mode][cfg.device & 63];
     if (o == 0) {
+        if (async && mode == kPeelRepair &&
+            cudaFuncSetAttribute(fns[async][mode], cudaFuncAttributePreferredSharedMemoryCarveout,
+                                 kTailCarveout) != cudaSuccess)
+            return -3;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, fns[async][mode], kThreads, 0) !=
                 cudaSuccess ||
             o <= 0)

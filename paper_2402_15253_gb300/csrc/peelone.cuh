@@ -54,7 +54,7 @@ namespace peel {
 // then (asynchronous levels) the static frontier's small and chunk counts
 enum : int {
     L_QS = 0, L_QB = 1, L_KEPT = 2 /* 2..4 */, L_MIN = 5 /* 5..7 */, L_FS = 8 /* 8..10 */,
-    L_FB = 11 /* 11..13 */, L_FA = 14 /* 14..16: the static frontier's arcs, capped per warp */, L_DMAX = 17
+    L_FB = 11 /* 11..13 */, L_FA = 14 /* 14..16: the static frontier's arcs, capped */, L_DMAX = 17
 };
 
 constexpr int kScanItems = 4;   // residual-list entries per thread per scan step
@@ -489,14 +489,14 @@ __device__ __forceinline__ void warp_push_ranges(bool pred, int rs, int d, bool 
                                                  unsigned *counter, unsigned cap, Ctrl *ctl,
                                                  int chunk)
 {
+    if (!__any_sync(kFull, pred)) return;
     unsigned nch = pred ? (unsigned)((d + chunk - 1) / chunk) : 0u;
     const unsigned pos = warp_reserve(counter, nch);
     if (nch > 0 && (unsigned long long)pos + nch > cap) {
         set_error(ctl, kErrNotConverged);
         nch = 0;
     }
-    if (__any_sync(kFull, nch > 0))
-        warp_fill<true>(nch, pos, list, RangeEntry(rs, d, chunk, guard));
+    warp_fill<true>(nch, pos, list, RangeEntry(rs, d, chunk, guard));
 }
 
 // One warp walks the arcs [s, t) of col_idx (a range entry).
@@ -632,7 +632,10 @@ __device__ bool run_async(const Params<Off> &p, GridDom &dom, unsigned *s_tmp,
     // ticket index of this warp: consecutive tickets go to different CTAs
     const unsigned tix = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
     __shared__ int s_loc[kThreads / 32][32];   // local slots of each warp
+    __shared__ unsigned s_front;               // arcs of the scan's frontier, this CTA's share
     __shared__ unsigned s_busy;                // warps of this CTA that are not idle
+    if (threadIdx.x == 0) s_front = 0;
+    __syncthreads();
     __shared__ unsigned long long s_acc;       // walked by idle warps, not yet in `done`
 
     const int mode = kTail ? ld_relaxed(&p.tail->mode) : (int)kTailFresh;
@@ -764,12 +767,15 @@ __device__ bool run_async(const Params<Off> &p, GridDom &dom, unsigned *s_tmp,
                 warp_push_chunks(c[j] == k && d[j] > p.tn.small_deg, v[j], d[j], p.fb,
                                  &live[L_FB + slot], p.qb_cap, ctl, p.tn.chunk);
         }
-        if (kTail && !last) {   // rare: most threads find no vertex at k
-            const unsigned a = (unsigned)min(front_arcs, 1ull << 18);
-            const unsigned sum = __reduce_add_sync(kFull, a);
-            if (lane == 0 && sum) atomicAdd(&live[L_FA + slot], min(sum, 1u << 18));
+        if (kTail && !last) {
+            const unsigned sum = __reduce_add_sync(kFull, (unsigned)min(front_arcs, 1ull << 18));
+            if (lane == 0 && sum) atomicAdd(&s_front, min(sum, 1u << 18));
         }
-        block_max_to(mx, &live[L_MIN + slot], s_tmp);
+        block_max_to(mx, &live[L_MIN + slot], s_tmp);   // (a CTA barrier)
+        if (kTail && !last && threadIdx.x == 0 && s_front) {   // one atomic per CTA
+            atomicAdd(&live[L_FA + slot], s_front);
+            s_front = 0;
+        }
         // the last arrival deals out the level's first tickets by moving the
         // heads past them
         if (!dom.sync_hook(set_heads)) return true;

@@ -526,13 +526,14 @@ __device__ __forceinline__ void warp_push_chunks(bool pred, int v, long long d, 
                                                  unsigned *counter, unsigned cap, Ctrl *ctl,
                                                  int chunk)
 {
+    if (!__any_sync(kFull, pred)) return;
     unsigned nch = pred ? (unsigned)((d + chunk - 1) / chunk) : 0u;
     const unsigned pos = warp_reserve(counter, nch);
     if (nch > 0 && (unsigned long long)pos + nch > cap) {
         set_error(ctl, kErrNotConverged);
         nch = 0;
     }
-    if (__any_sync(kFull, nch > 0)) warp_fill<kRelaxedStores>(nch, pos, list, ChunkEntry(v));
+    warp_fill<kRelaxedStores>(nch, pos, list, ChunkEntry(v));
 }
 
 // Default number of arcs a lane issues per step of expand(): their loads and
