@@ -151,8 +151,9 @@ int pico_validate_graph_i64(const int64_t *row_ptr, const int32_t *col_idx, int6
  *   total_vertices, total_arcs: must equal vtx_off[G] and arc_off[G] (the
  *     host cannot read device memory without synchronising).
  *   out_core: device int32, vtx_off[G] entries, each graph's coreness.
- * One CTA solves one graph at a time, largest graphs first; a graph needs
- * fewer than 2^31 arcs. G == 0 is a no-op.
+ * Graphs are taken largest first, by one CTA or one thread-block cluster at a
+ * time, according to their size; a graph needs fewer than 2^31 arcs. G == 0 is a
+ * no-op.
  */
 int pico_coreness_batched(const int64_t *vtx_off, const int64_t *arc_off, int32_t G,
                           const int32_t *row_ptr, const int32_t *col_idx,
@@ -274,10 +275,13 @@ typedef struct {
     int64_t rounds;      /* HistoCore: SumHisto/UpdateHisto rounds */
     int64_t frontier;    /* HistoCore: sum over rounds of |V_cnt| */
     int64_t barriers;    /* grid-wide barriers executed */
-    int64_t arcs;        /* PeelOne: adjacency entries read by the expansion phases;
+    int64_t arcs;        /* PeelOne: adjacency entries of the vertices that Alg. 4
+                            expands (a run ends early once every vertex is queued);
                             HistoCore: arcs of InitHisto plus, per round, the arcs of the
                             changed vertices (what Alg. 6 scans, in either direction) */
-    int64_t atomics;     /* atomic read-modify-writes on core[] or histo[] */
+    int64_t atomics;     /* atomic read-modify-writes on core[] or histo[]; the
+                            shared-memory and cluster forms of PeelOne count the
+                            successful decrements */
     int64_t slots;       /* HistoCore: histogram slots read by SumHisto */
     int64_t blocks;      /* CTAs of the persistent launch */
     int64_t scanned;     /* PeelOne: residual-list entries read, summed over scans */
@@ -289,7 +293,9 @@ typedef struct {
     /* Device time (ns) and count per phase kind, measured by CTA 0 from one
        grid barrier to the next: [0] init, [1] PeelOne residual scan,
        [2..4] PeelOne frontier waves with < 64 work units / fewer units than
-       warps / more, [5] InitHisto, [6] SumHisto, [7] UpdateHisto. */
+       warps / more, [5] InitHisto, [6] SumHisto, [7] UpdateHisto. [3] also
+       holds the launches that peel in one CTA or one cluster, each as one
+       phase, and [4] the asynchronous levels of the grid kernel. */
     int64_t phase_ns[8];
     int64_t phase_count[8];
 } pico_stats;
@@ -325,10 +331,10 @@ int pico_selftest_wait_timeout(int limit_ms, pico_stream_t stream);
  * autotuner, paper_2402_15253_gb300/autotune.py): vertices of degree at most
  * small_deg (32..256) are batched 32 per warp; larger ones are split into
  * chunks of `chunk` arcs (64..4096), one per warp; batched_threads (256 or
- * 512) is the CTA size of the batched kernel, where a graph with at least
- * 2^cluster_log2 arcs (10..62; 62 disables clusters) is solved by a cluster of
- * 8 CTAs and every other graph by one CTA. Applies to later calls on the
- * device; defaults 32, 256, 512, 21. Results never depend on these values,
+ * 512) is the CTA size of the batched HistoCore kernel, where a graph with at
+ * least 2^cluster_log2 arcs (10..62; 62 disables clusters) is solved by a cluster
+ * of 8 CTAs and every other graph by one CTA (batched PeelOne chooses by the
+ * number of vertices). Applies to later calls on the device; defaults 32, 256, 512, 21. Results never depend on these values,
  * only the speed does.
  */
 int pico_set_tuning(int small_deg, int chunk, int batched_threads, int cluster_log2);

@@ -10,11 +10,14 @@
 //   tiny    n <= kTinyVertices: CTAs of kTinyThreads threads, eight per SM, so
 //           that one graph's barriers and chains overlap the others'.
 //   middle  n <= kLocalSlots: one CTA of kWideThreads threads per graph.
-//   large   the rest: a cluster of kPeelCtas CTAs per graph; a graph that does
-//           not fit their shared memory either is peeled in global memory
+//   large   n <= kPeelCtas * kLocalSlots: a cluster of kPeelCtas CTAs per graph.
+//   huge    the rest: a cluster of kClusterCtas CTAs per graph, in global memory
 //           (peel::run over the cluster).
 // Middle and large graphs share one launch: clusters first take the large
-// graphs, then each CTA takes middle ones; the tiny ones are a second launch.
+// graphs, then each CTA takes middle ones. It does not wait for the launch of
+// the huge graphs before it, which leaves SMs free (24 graphs of 1 M vertices and
+// 488 smaller ones: 27.2 ms one after the other, 23.7 ms side by side). The tiny
+// graphs are the last launch, which waits for both.
 //
 // HistoCore runs the single-graph body (histo::run) in two phases: graphs of
 // at least 2^cluster_log2 arcs (a tuning value) by clusters of kClusterCtas
@@ -47,8 +50,8 @@ constexpr size_t kTinySmem = 26 * 1024;         // eight CTAs share an SM's 228 
 static_assert(kTinySmem >= 16 * kTinyVertices / 2 + 4096, "row offsets of a tiny graph must fit");
 
 // control words of the batched launch (in Ctrl::live): tickets of the classes,
-// the number of graphs in the first class, and in the first two
-enum : int { B_SMALL = 0, B_LARGE = 1, B_NLARGE = 2, B_TINY = 3, B_NMIDDLE = 4 };
+// and where the classes end in the schedule
+enum : int { B_SMALL = 0, B_LARGE = 1, B_NLARGE = 2, B_TINY = 3, B_NMIDDLE = 4, B_HUGE = 5, B_NHUGE = 6 };
 
 struct BatchParams {
     const long long *vtx_off, *arc_off;
@@ -69,24 +72,26 @@ __device__ __forceinline__ int size_bucket(long long m)
     return m <= 0 ? 0 : 64 - __clzll(m);
 }
 
-// Class of a graph: 2 (listed first) to 0. PeelOne: by where its residual
-// degrees fit; HistoCore: by its arcs (class 1 is not used).
+// Class of a graph: 3 (listed first) to 0. PeelOne: by where its residual
+// degrees fit; HistoCore: by its arcs (classes 2 and 0).
 __device__ __forceinline__ int graph_class(long long n, long long m, int algo, int cluster_log2)
 {
     if (algo != 0) return size_bucket(m) > cluster_log2 ? 2 : 0;
-    return n > peel::kLocalSlots ? 2 : (n > kTinyVertices ? 1 : 0);
+    return n > (long long)kPeelCtas * peel::kLocalSlots ? 3
+           : n > peel::kLocalSlots                      ? 2
+                                                        : (n > kTinyVertices ? 1 : 0);
 }
 
 // Lists the graphs by class and decreasing arc-count bucket (one CTA) and
-// records how many lead the list in class 2, and in classes 2 and 1 (bucket b
-// holds arc counts in [2^(b-1), 2^b)).
+// records where classes 3, 2 and 1 end in the list (bucket b holds arc counts
+// in [2^(b-1), 2^b)).
 __global__ void __launch_bounds__(1024)
     schedule_kernel(const long long *vtx_off, const long long *arc_off, int G, int *order, Ctrl *ctl,
                     int algo, int cluster_log2)
 {
-    __shared__ unsigned cnt[3 * kBuckets];
-    __shared__ unsigned start[3 * kBuckets];
-    if (threadIdx.x < 3 * kBuckets) cnt[threadIdx.x] = 0;
+    __shared__ unsigned cnt[4 * kBuckets];
+    __shared__ unsigned start[4 * kBuckets];
+    if (threadIdx.x < 4 * kBuckets) cnt[threadIdx.x] = 0;
     __syncthreads();
     auto key = [&](int g) {
         const long long n = vtx_off[g + 1] - vtx_off[g], m = arc_off[g + 1] - arc_off[g];
@@ -96,9 +101,10 @@ __global__ void __launch_bounds__(1024)
     __syncthreads();
     if (threadIdx.x == 0) {
         unsigned run = 0;
-        for (int b = 3 * kBuckets - 1; b >= 0; --b) {
+        for (int b = 4 * kBuckets - 1; b >= 0; --b) {
             start[b] = run;
             run += cnt[b];
+            if (b == 3 * kBuckets) ctl->live.w[B_NHUGE] = run;
             if (b == 2 * kBuckets) ctl->live.w[B_NLARGE] = run;
             if (b == kBuckets) ctl->live.w[B_NMIDDLE] = run;
         }
@@ -222,11 +228,16 @@ __device__ __forceinline__ peel::LocalParams<int> local_params(const BatchParams
             bp.core + v0,   bp.qs + v0, bp.ctl};
 }
 
-// PeelOne, large and middle graphs.
-__global__ void __launch_bounds__(kWideThreads, 1) batched_peel_kernel(BatchParams bp)
+// PeelOne, huge graphs: one cluster per graph. Bound by the latency of L2 atomics
+// and of the cluster barriers; 8 CTAs of 512 threads, two to an SM, keep twice the
+// warps that 4 CTAs of 1,024 have, and leave room for a second graph beside them
+// (one R-MAT graph of 2^20 vertices and 31 M arcs: 35 -> 16.5 ms; 24 of them and
+// 488 smaller graphs: 41.8 -> 23.7 ms).
+__global__ void __launch_bounds__(512, 2) batched_huge_kernel(BatchParams bp)
 {
     namespace cg = cooperative_groups;
-    extern __shared__ __align__(16) char smem[];
+    // the next launch may start: it shares nothing with this one
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     __shared__ __align__(16) unsigned s_live[kLiveWords];
     __shared__ unsigned s_snap[kLiveWords + 1];
     __shared__ unsigned s_tmp[256];
@@ -236,34 +247,59 @@ __global__ void __launch_bounds__(kWideThreads, 1) batched_peel_kernel(BatchPara
     if (threadIdx.x < kStCount) st[threadIdx.x] = 0;
     __syncthreads();
     cg::cluster_group cluster = cg::this_cluster();
-    const unsigned crank = cluster.block_rank();
+    const unsigned crank = cluster.block_rank(), csize = cluster.num_blocks();
     PhaseClock clk;
     unsigned long long arcs = 0, atomics = 0, slots = 0, pulled = 0, extra = 0;
+    const int nhuge = (int)ld_relaxed(&bp.ctl->live.w[B_NHUGE]);
+    ClusterDom dom{bp.ctl, s_live, cluster.map_shared_rank(s_live, 0), s_snap, crank, csize, 0u};
+    int *ticket0 = cluster.map_shared_rank(&s_ticket, 0);
+    for (;;) {
+        if (crank == 0 && threadIdx.x == 0) {
+            const int t = (int)atomicAdd(&bp.ctl->live.w[B_HUGE], 1u);
+            s_ticket = (t < nhuge && status_of(bp.ctl) == 0) ? t : -1;
+        }
+        cluster.sync();
+        const int t = *ticket0;
+        cluster.sync();
+        if (t < 0) break;
+        solve_graph<0>(bp, bp.order[t], dom, s_tmp, st, clk, arcs, atomics, slots, pulled, extra);
+    }
+    block_sum_to(arcs, &bp.ctl->stats[kStArcs], s_red);
+    block_sum_to(atomics, &bp.ctl->stats[kStAtomics], s_red);
+    block_sum_to(extra, &bp.ctl->stats[kStExtra], s_red);
+    fold_block(bp.ctl, st);
+    cluster.sync();   // no CTA leaves while another may still read its shared memory
+}
 
+// PeelOne, large and middle graphs.
+__global__ void __launch_bounds__(kWideThreads, 1) batched_peel_kernel(BatchParams bp)
+{
+    namespace cg = cooperative_groups;
+    extern __shared__ __align__(16) char smem[];
+    __shared__ unsigned long long st[kStCount];
+    __shared__ int s_ticket;
+    if (threadIdx.x < kStCount) st[threadIdx.x] = 0;
+    __syncthreads();
+    cg::cluster_group cluster = cg::this_cluster();
+    const unsigned crank = cluster.block_rank();
+    const int nhuge = (int)ld_relaxed(&bp.ctl->live.w[B_NHUGE]);
     const int nlarge = (int)ld_relaxed(&bp.ctl->live.w[B_NLARGE]);
     const int nmiddle = (int)ld_relaxed(&bp.ctl->live.w[B_NMIDDLE]);
     {   // large graphs, one cluster per graph
-        ClusterDom dom{bp.ctl, s_live, cluster.map_shared_rank(s_live, 0), s_snap, crank, kPeelCtas,
-                       0u};
         int *ticket0 = cluster.map_shared_rank(&s_ticket, 0);
         for (;;) {
             if (crank == 0 && threadIdx.x == 0) {
-                const int t = (int)atomicAdd(&bp.ctl->live.w[B_LARGE], 1u);
+                const int t = nhuge + (int)atomicAdd(&bp.ctl->live.w[B_LARGE], 1u);
                 s_ticket = (t < nlarge && status_of(bp.ctl) == 0) ? t : -1;
             }
             cluster.sync();
             const int t = *ticket0;
             cluster.sync();
             if (t < 0) break;
-            const int g = bp.order[t];
-            if (bp.vtx_off[g + 1] - bp.vtx_off[g] <= (long long)kPeelCtas * peel::kLocalSlots) {
-                const peel::LocalParams<int> p = local_params(bp, g);
-                const peel::LocalStats s =
-                    peel::run_local<int, peel::LocalWide, true>(p, smem, crank, kPeelCtas);
-                if (crank == 0 && threadIdx.x == 0) peel::add_stats(st, s, p.n, p.m);
-            } else {
-                solve_graph<0>(bp, g, dom, s_tmp, st, clk, arcs, atomics, slots, pulled, extra);
-            }
+            const peel::LocalParams<int> p = local_params(bp, bp.order[t]);
+            const peel::LocalStats s =
+                peel::run_local<int, peel::LocalWide, true>(p, smem, crank, kPeelCtas);
+            if (crank == 0 && threadIdx.x == 0) peel::add_stats(st, s, p.n, p.m);
         }
     }
     for (;;) {   // middle graphs, one CTA per graph
@@ -281,11 +317,11 @@ __global__ void __launch_bounds__(kWideThreads, 1) batched_peel_kernel(BatchPara
         if (threadIdx.x == 0) peel::add_stats(st, s, p.n, p.m);
         __syncthreads();
     }
-    block_sum_to(arcs, &bp.ctl->stats[kStArcs], s_red);
-    block_sum_to(atomics, &bp.ctl->stats[kStAtomics], s_red);
-    block_sum_to(extra, &bp.ctl->stats[kStExtra], s_red);
     fold_block(bp.ctl, st);
     cluster.sync();   // no CTA leaves while another may still read its shared memory
+    // this launch ends after the one before it, so that what follows waits for
+    // both; one CTA waits, the others give their SMs to other streams
+    if (blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // PeelOne, tiny graphs; the second launch of a batch, which publishes its
@@ -320,12 +356,14 @@ __global__ void __launch_bounds__(kTinyThreads, 8) batched_tiny_kernel(BatchPara
 
 // Launches a kernel over a persistent grid of clusters: every cluster that is
 // resident at once, but no more than `need`. occ: the kernel's cached number
-// of resident clusters (0: not known yet).
+// of resident clusters (0: not known yet). beside: the launch may run beside the
+// one before it on the stream.
 cudaError_t launch_clusters(const void *fn, int cluster, int threads, size_t smem, int sms,
-                            long long need, int &occ, void **args, cudaStream_t stream)
+                            long long need, int &occ, void **args, cudaStream_t stream,
+                            bool beside = false)
 {
     cudaLaunchConfig_t lc = {};
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = cluster;
     attr[0].val.clusterDim.y = 1;
@@ -347,6 +385,11 @@ cudaError_t launch_clusters(const void *fn, int cluster, int threads, size_t sme
         if (occ <= 0) return cudaErrorLaunchOutOfResources;
     }
     lc.gridDim = dim3(cluster * (unsigned)std::min<long long>(need, occ));
+    if (beside) {
+        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[1].val.programmaticStreamSerializationAllowed = 1;
+        lc.numAttrs = 2;
+    }
     return cudaLaunchKernelExC(&lc, fn, args);
 }
 
@@ -408,14 +451,19 @@ int launch_batched(const int64_t *vtx_off, const int64_t *arc_off, int G, const 
 
     const int dev = cfg.device & 63;
     if (algo == 0) {
-        static int occ_wide[64] = {}, occ_tiny[64] = {};
+        static int occ_huge[64] = {}, occ_wide[64] = {}, occ_tiny[64] = {};
         void *args[] = {&bp, &last};
-        // graphs the launch can hold (its grids need no more CTAs than that)
+        // graphs of a class the batch can hold (its grid needs no more clusters)
+        const long long huge =
+            std::min<long long>(G, total_n / ((long long)kPeelCtas * peel::kLocalSlots + 1));
+        if (huge > 0 && launch_clusters((const void *)batched_huge_kernel, kClusterCtas, 512, 0,
+                                        cfg.sms, huge, occ_huge[dev], args, stream) != cudaSuccess)
+            return -3;
         const long long wide = std::min<long long>(G, total_n / (kTinyVertices + 1));
         if (wide > 0 &&
             launch_clusters((const void *)batched_peel_kernel, kPeelCtas, kWideThreads,
                             peel::kLocalSmem, cfg.sms,
-                            wide, occ_wide[dev], args, stream) != cudaSuccess)
+                            wide, occ_wide[dev], args, stream, huge > 0) != cudaSuccess)
             return -3;
         if (launch_clusters((const void *)batched_tiny_kernel, 1, kTinyThreads,
                             kTinySmem, cfg.sms * 8, G,

@@ -79,7 +79,6 @@ struct TailState {
     unsigned cur;       // ... in res1 (1) or res0
     unsigned lo, hi;
     unsigned spilled;   // cluster kernel: entries listed in fs during a wave
-    int skewed;         // the grid kernel may hand levels over
     int published;      // the run's status and statistics are out (method selection)
 };
 

@@ -150,3 +150,35 @@ def test_batched_forms(pico, name, sizes):
     assert st["kmax"] == int(want.max())
     assert st["arcs"] == int(pb.arc_off[-1])
     assert st["atomics"] - st["extra"] == int(pb.arc_off[-1]) - int(want.sum())
+
+
+def test_batched_forms_replayed(pico):
+    """Graphs of every size class recorded in one CUDA graph, where the launch
+    for the largest runs beside the next one; every replay gives the oracle's
+    coreness."""
+    graphs = [gg.er_graph(CLUSTER_SLOTS + 9, 900000, 95), ring_of(300000, 5), gg.star_graph(90000),
+              gg.er_graph(30000, 120000, 96), gg.complete_graph(60)]
+    pb = gg.pack_graphs(graphs)
+    want = oracle.bz_coreness_batched(pb.vtx_off, pb.arc_off, pb.row_ptr, pb.col_idx)
+    tv, ta = int(pb.vtx_off[-1]), int(pb.arc_off[-1])
+    d = [t.cuda() for t in (pb.vtx_off, pb.arc_off, pb.row_ptr, pb.col_idx)]
+    out = torch.full((tv,), -1, dtype=torch.int32, device="cuda")
+    s, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+
+    def call():
+        return pico.pico_coreness_batched(d[0], d[1], len(graphs), d[2], d[3], tv, ta, out,
+                                          pico.ALGOS["peelone"], s)
+
+    s.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(s):
+        assert call() == pico.PICO_OK
+        s.synchronize()
+        with torch.cuda.graph(graph, stream=s):
+            assert call() == pico.PICO_OK
+    for _ in range(2):
+        torch.cuda.synchronize()
+        out.fill_(-1)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert pico.pico_last_device_status() == pico.PICO_OK
+        assert np.array_equal(out.cpu().numpy(), want)
