@@ -183,7 +183,11 @@ struct TailPeel {
     }
 
     // Cluster barrier after which every CTA knows every CTA's queue length, and
-    // the sums and minima of the rest.
+    // the sums and minima of the rest. What the next phase counts from zero is
+    // cleared here, after it was sent and before the CTA arrives: a warp that has
+    // left the barrier may count at once (a small wave has no CTA barrier of its
+    // own). That is the count of the other queue buffer (the wave just walked it), the
+    // scan's counters and, after a scan, the near buffer it read.
     __device__ __forceinline__ TailTotals exchange(bool of_scan)
     {
         __syncthreads();
@@ -201,6 +205,12 @@ struct TailPeel {
             asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr + 16), "r"(near) : "memory");
         }
         __syncwarp();
+        if (threadIdx.x == 0) {
+            sh.qn[qb ^ 1u] = 0;
+            sh.kept = sh.overflow = 0;
+            sh.vmin = INT_MAX;
+            if (of_scan) sh.near_n[nb ^ 1u] = 0;
+        }
         asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
         asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
         uint4 a = make_uint4(0, (unsigned)INT_MAX, 0, 0);
@@ -454,19 +464,14 @@ struct TailPeel {
             } else {
                 left -= t.queued;
             }
+            // a near list that overflowed is not read: the next scan is of the
+            // residual list, and its exchange clears the buffer
             if (t.overflow) hi = k + 1;
-            if (threadIdx.x == 0) {
-                sh.near_n[nb ^ 1u] = 0;   // the next scan's buffer
-                if (t.overflow) sh.near_n[nb] = 0;
-                sh.kept = sh.overflow = 0;
-                sh.vmin = INT_MAX;
-            }
             if (lead) {
                 ++st[kStScans];
                 st[kStScanned] += full ? t.kept + t.queued : t.near_max;
             }
             if (t.queued == 0) {   // empty level
-                __syncthreads();
                 if (t.vmin != INT_MAX) k = t.vmin;
                 else if (full) break;   // nothing is left
                 else k = hi;
@@ -477,6 +482,7 @@ struct TailPeel {
                 if ((unsigned long long)k > st[kStKmax]) st[kStKmax] = (unsigned long long)k;
             }
             // ---- waves
+            bool lost = false;   // a wave's additions to the near list did not fit
             while (t.queued > 0 && left > 0) {
                 const unsigned b = qb, own = min(sh.x[par ^ 1u][rank][0].x, (unsigned)kTailQueue);
                 settle(b, own);
@@ -499,7 +505,7 @@ struct TailPeel {
                 listed = beyond;
                 t = exchange(false);
                 left -= t.queued;
-                if (threadIdx.x == 0) sh.qn[b] = 0;   // the buffer of the wave after the next
+                lost |= t.overflow;
                 if (lead) ++st[kStSubrounds];
             }
             if (mode == kTailPending) break;
@@ -507,13 +513,7 @@ struct TailPeel {
                 settle(qb, min(sh.x[par ^ 1u][rank][0].x, (unsigned)kTailQueue));
                 break;
             }
-            if (t.overflow) hi = k + 1;
-            __syncthreads();   // every warp has left the exchange
-            if (threadIdx.x == 0 && t.overflow) {
-                sh.near_n[nb] = 0;
-                sh.overflow = 0;
-            }
-            __syncthreads();
+            if (lost) hi = k + 1;
             ++k;
         }
         if (mode == kTailDone) {

@@ -1,0 +1,89 @@
+"""PeelOne's light levels on one cluster, between launches of the grid kernel.
+
+Every graph here is handed over, which the phase counts show: "wave_mid" counts
+the launches that peeled on the cluster, "init" the initialisation and every wave
+that the grid kernel took back. Results and counts of work are the
+oracle's.
+"""
+import numpy as np
+import pytest
+import torch
+
+import graphgen as gg
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def pico():
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2402_15253_gb300 as p
+    torch.cuda.set_device(0)
+    return p
+
+
+def peel(pico, g, off):
+    """Compares with the oracle; returns (cluster launches, waves taken back)."""
+    rp, ci = g.numpy()
+    want = oracle.bz_coreness(rp, ci)
+    _, ost = oracle.peelone(rp, ci)
+    got = pico.coreness(g.row_ptr.to("cuda", dtype=off), g.col_idx.cuda(), "peelone").cpu().numpy()
+    st = pico.pico_get_stats()
+    assert np.array_equal(got, want), f"{int((got != want).sum())} vertices differ"
+    assert st["levels"] == ost["levels"] and st["kmax"] == ost["kmax"]
+    assert st["arcs"] == ost["arcs_scanned"]
+    assert st["atomics"] - st["extra"] == ost["decrements"]
+    ph = st["phases"]
+    return ph.get("wave_mid", {"count": 0})["count"], ph["init"]["count"] - 1
+
+
+def circulant(n, reach, first=0):
+    """Pairs of n vertices from `first` on, each joined to the next `reach`."""
+    i = torch.arange(n, dtype=torch.int64).repeat_interleave(reach)
+    d = torch.arange(1, reach + 1, dtype=torch.int64).repeat(n)
+    return first + i, first + (i + d) % n
+
+
+def union(n, *pairs):
+    return gg.csr_from_pairs(torch.cat([p[0] for p in pairs]), torch.cat([p[1] for p in pairs]), n)
+
+
+def star(hub, ends):
+    return torch.full_like(ends, hub), ends
+
+
+def strips(count):
+    """`count` strips of 500 squares of distinct widths over one dense part: each
+    peels from its end in waves of a few vertices, many in a row."""
+    core = 60000
+    pairs = [circulant(core, 24), star(0, torch.arange(30, 6000))]
+    at = core
+    for c in range(count):
+        w = 4 + c
+        ids = at + torch.arange(500 * w, dtype=torch.int64).view(500, w)
+        pairs.append((ids[:-1].reshape(-1), ids[1:].reshape(-1)))
+        # each vertex is held by w others of its strip's next column
+        for s in range(1, w):
+            pairs.append((ids[:-1].reshape(-1), ids[1:].roll(s, 1).reshape(-1)))
+        pairs.append((ids[-1].repeat_interleave(30), torch.arange(30).repeat(w) + 100 * c))
+        at += 500 * w
+    return union(at, *pairs)
+
+
+def near_overflow():
+    """More residual vertices inside the first window than the near lists hold."""
+    n = 300000
+    gen = torch.Generator().manual_seed(7)
+    return union(n, (torch.randint(n, (10 * n,), generator=gen), torch.randint(n, (10 * n,), generator=gen)),
+                 star(5, torch.arange(6, 9000)))
+
+
+@pytest.mark.parametrize("off", [torch.int32, torch.int64], ids=["int32", "int64"])
+@pytest.mark.parametrize("make", [lambda: strips(20), near_overflow], ids=["strips", "near-overflow"])
+def test_consecutive_waves(pico, make, off):
+    g = make()
+    for _ in range(3):
+        launches, _ = peel(pico, g, off)
+        assert launches >= 1
