@@ -163,6 +163,23 @@ __device__ __forceinline__ void solve_graph(const BatchParams &bp, int g, Dom &d
     }
 }
 
+// The CTA's next graph: a place in the schedule from `first` up to `end`, or -1
+// when there is none left or the call has failed. One thread decides for all: an
+// error that another CTA records meanwhile would otherwise send some warps out of
+// the loop and leave the others waiting for them.
+__device__ __forceinline__ int next_ticket(const BatchParams &bp, int word, int first, int end,
+                                           int *s_ticket)
+{
+    if (threadIdx.x == 0) {
+        const int t = first + (int)atomicAdd(&bp.ctl->live.w[word], 1u);
+        *s_ticket = (t < end && status_of(bp.ctl) == 0) ? t : -1;
+    }
+    __syncthreads();
+    const int t = *s_ticket;
+    __syncthreads();
+    return t;
+}
+
 // HistoCore.
 template <int Threads>
 __global__ void __launch_bounds__(Threads, 512 / Threads * 2)
@@ -204,11 +221,8 @@ __global__ void __launch_bounds__(Threads, 512 / Threads * 2)
     {
         CtaDom dom{bp.ctl, s_live, s_snap, 0u};
         for (;;) {
-            if (threadIdx.x == 0) s_ticket = nlarge + (int)atomicAdd(&bp.ctl->live.w[B_SMALL], 1u);
-            __syncthreads();
-            const int t = s_ticket;
-            __syncthreads();
-            if (t >= bp.G || status_of(bp.ctl) != 0) break;
+            const int t = next_ticket(bp, B_SMALL, nlarge, bp.G, &s_ticket);
+            if (t < 0) break;
             solve_graph<1>(bp, bp.order[t], dom, s_tmp, st, clk, arcs, atomics, slots, pulled, extra);
             __syncthreads();
         }
@@ -303,11 +317,8 @@ __global__ void __launch_bounds__(kWideThreads, 1) batched_peel_kernel(BatchPara
         }
     }
     for (;;) {   // middle graphs, one CTA per graph
-        if (threadIdx.x == 0) s_ticket = nlarge + (int)atomicAdd(&bp.ctl->live.w[B_SMALL], 1u);
-        __syncthreads();
-        const int t = s_ticket;
-        __syncthreads();
-        if (t >= nmiddle || status_of(bp.ctl) != 0) break;
+        const int t = next_ticket(bp, B_SMALL, nlarge, nmiddle, &s_ticket);
+        if (t < 0) break;
         const peel::LocalParams<int> p = local_params(bp, bp.order[t]);
         const bool rows = peel::local_smem_bytes<peel::LocalWide>(p.n, peel::kKeepRows) <=
                           peel::kLocalSmem;
@@ -335,11 +346,8 @@ __global__ void __launch_bounds__(kTinyThreads, 8) batched_tiny_kernel(BatchPara
     __syncthreads();
     const int nmiddle = (int)ld_relaxed(&bp.ctl->live.w[B_NMIDDLE]);
     for (;;) {
-        if (threadIdx.x == 0) s_ticket = nmiddle + (int)atomicAdd(&bp.ctl->live.w[B_TINY], 1u);
-        __syncthreads();
-        const int t = s_ticket;
-        __syncthreads();
-        if (t >= bp.G || status_of(bp.ctl) != 0) break;
+        const int t = next_ticket(bp, B_TINY, nmiddle, bp.G, &s_ticket);
+        if (t < 0) break;
         const peel::LocalParams<int> p = local_params(bp, bp.order[t]);
         if (p.n <= 0) continue;
         const bool whole = peel::local_smem_bytes<peel::LocalTiny>(p.n, peel::kKeepGraph, p.m) <=
