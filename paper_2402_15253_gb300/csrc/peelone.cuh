@@ -633,12 +633,16 @@ __device__ bool run_async(const Params<Off> &p, GridDom &dom, unsigned *s_tmp,
     __shared__ int s_loc[kThreads / 32][32];   // local slots of each warp
     __shared__ unsigned s_front;               // arcs of the scan's frontier, this CTA's share
     __shared__ unsigned s_busy;                // warps of this CTA that are not idle
-    if (threadIdx.x == 0) s_front = 0;
-    __syncthreads();
     __shared__ unsigned long long s_acc;       // walked by idle warps, not yet in `done`
-
-    const int mode = kTail ? ld_relaxed(&p.tail->mode) : (int)kTailFresh;
-    if (kTail && (mode == kTailDone || status_of(ctl) != 0)) return true;
+    __shared__ int s_mode;
+    if (threadIdx.x == 0) {   // for all: another CTA's wait may run out meanwhile
+        s_front = 0;
+        s_mode = kTailFresh;
+        if (kTail) s_mode = status_of(ctl) != 0 ? (int)kTailDone : ld_relaxed(&p.tail->mode);
+    }
+    __syncthreads();
+    const int mode = s_mode;
+    if (mode == kTailDone) return true;
     // init: work = degree, isolated vertices get 0, residual list, queue
     // slots empty, control lines zero
     if (mode == kTailFresh) {

@@ -38,7 +38,7 @@ def reads(name):
 ONE_THREAD = re.compile(r"if \(.*(threadIdx\.x == 0|lane == 0).*\)$")
 
 
-@pytest.mark.parametrize("name", ["batched.cu"])
+@pytest.mark.parametrize("name", ["batched.cu", "peelone.cuh"])
 def test_one_thread_reads_the_status(name):
     found = reads(name)
     assert found
