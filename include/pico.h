@@ -327,6 +327,16 @@ int pico_get_trace(pico_stream_t stream, int64_t *out, int cap);
 int pico_selftest_wait_timeout(int limit_ms, pico_stream_t stream);
 
 /*
+ * Self-test of how a call of several launches reports an error (PeelOne's
+ * launches hand levels over to one another). A launch of 64 CTAs records
+ * PICO_ERR_TIMEOUT and 20 of its CTAs leave without finishing, as when a wait runs
+ * out while a level is handed over; a launch of 16 CTAs then ends the call. Synchronises
+ * `stream` and returns the device status that was reported: PICO_ERR_TIMEOUT when
+ * the error is not lost. Clears the sticky status before and after.
+ */
+int pico_selftest_handover(pico_stream_t stream);
+
+/*
  * Degree-class work assignment of the current device's kernels (set by the
  * autotuner, paper_2402_15253_gb300/autotune.py): vertices of degree at most
  * small_deg (32..256) are batched 32 per warp; larger ones are split into

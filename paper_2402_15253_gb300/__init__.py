@@ -159,6 +159,8 @@ def load(path: str = LIB_PATH) -> ctypes.CDLL:
     L.pico_get_histo_update.restype = i32
     L.pico_selftest_wait_timeout.argtypes = [i32, vp]
     L.pico_selftest_wait_timeout.restype = i32
+    L.pico_selftest_handover.argtypes = [vp]
+    L.pico_selftest_handover.restype = i32
     L.pico_get_trace.argtypes = [vp, vp, i32]
     L.pico_get_trace.restype = i32
     L.pico_coreness_noalloc.argtypes = [vp, vp, i64, i64, vp, vp, vp]
@@ -610,6 +612,10 @@ def pico_get_tuning() -> tuple:
 
 def pico_selftest_wait_timeout(limit_ms: int, stream=None) -> int:
     return load().pico_selftest_wait_timeout(limit_ms, _stream(stream))
+
+
+def pico_selftest_handover(stream=None) -> int:
+    return load().pico_selftest_handover(_stream(stream))
 
 
 def pico_version() -> int:

@@ -471,6 +471,20 @@ int pico_selftest_wait_timeout(int limit_ms, pico_stream_t stream)
     return pico_last_device_status(stream);
 }
 
+int pico_selftest_handover(pico_stream_t stream)
+{
+    DeviceState *d = nullptr;
+    int rc = device_state(&d);
+    if (rc != PICO_OK) return rc;
+    (void)pico_last_device_status(stream);   // start from a clean status
+    rc = pico::selftest_handover(d->last, (cudaStream_t)stream);
+    if (rc != 0) {
+        cudaGetLastError();
+        return rc == -2 ? PICO_ERR_OOM : PICO_ERR_CUDA;
+    }
+    return pico_last_device_status(stream);
+}
+
 int pico_set_tuning(int small_deg, int chunk, int batched_threads, int cluster_log2)
 {
     if (small_deg < pico::kMinSmallDeg || small_deg > pico::kMaxSmallDeg ||

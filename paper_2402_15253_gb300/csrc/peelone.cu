@@ -35,7 +35,7 @@ constexpr long long kLocalMaxArcs = 640 << 10;
 template <typename Off, int Mode, bool kAsync, bool kTail>
 __global__ void __launch_bounds__(kThreads, 2)
     peelone_kernel(peel::Params<Off> p, LastResult *last, unsigned long long limit_ns,
-                   long long m, bool final)
+                   long long m, int turn, bool final)
 {
     __shared__ unsigned s_snap[kLiveWords + 1];
     __shared__ unsigned s_tmp[128];
@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(kThreads, 2)
         p.ctl, last,
         Mode == kPeelRepair ? PICO_ALGO_PEELONE
                             : (Mode == kPeelCas ? PICO_ALGO_PEEL_CAS : PICO_ALGO_PEEL_ADDBACK),
-        st, kStCount);
+        st, kStCount, turn);
     if (kTail && published) p.tail->published = 1;
 }
 
@@ -83,7 +83,7 @@ __global__ void __launch_bounds__(kThreads, 2)
 // kernel (peel_tail.cuh).
 template <typename Off>
 __global__ void __launch_bounds__(peel::kTailThreads, 1)
-    peelone_tail_kernel(peel::Params<Off> p, LastResult *last, long long m, bool final)
+    peelone_tail_kernel(peel::Params<Off> p, LastResult *last, long long m, int turn, bool final)
 {
     extern __shared__ __align__(16) char smem[];
     __shared__ unsigned long long st[kStCount];
@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(peel::kTailThreads, 1)
     block_sum_to(tp.n_lowered, &p.ctl->stats[kStAtomics], s_red);
     if (over) {   // only CTA 0 counts levels and scans
         fold_kmax(p.ctl, st);
-        if (finish_block(p.ctl, last, PICO_ALGO_PEELONE, st, kStCount)) p.tail->published = 1;
+        if (finish_block(p.ctl, last, PICO_ALGO_PEELONE, st, kStCount, turn)) p.tail->published = 1;
     } else {
         fold_block(p.ctl, st);
     }
@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(kLocalThreads, 1)
     const peel::LocalStats s = peel::run_local<Off, peel::LocalWide, false, kKept>(p, smem, 0, 1);
     if (threadIdx.x == 0) peel::add_stats(st, s, p.n, p.m);
     clk.end(st, kPhWaveMid, (unsigned)s.waves);
-    finish_block(p.ctl, last, PICO_ALGO_PEELONE, st, kStCount);
+    finish_block(p.ctl, last, PICO_ALGO_PEELONE, st, kStCount, tail ? 1 : 0);
 }
 
 // Sets a kernel's dynamic shared memory limit (and non-portable cluster size)
@@ -157,7 +157,7 @@ bool prepare_kernel(const void *fn, size_t smem, bool wide_cluster, bool &ready)
 
 template <typename Off>
 cudaError_t launch_tail(peel::Params<Off> &p, long long m, LastResult *last, cudaStream_t stream,
-                        int device, bool final)
+                        int device, int turn, bool final)
 {
     static bool ready[64] = {};
     const void *fn = (const void *)peelone_tail_kernel<Off>;
@@ -179,7 +179,7 @@ cudaError_t launch_tail(peel::Params<Off> &p, long long m, LastResult *last, cud
     lc.stream = stream;
     lc.attrs = attr;
     lc.numAttrs = 1;
-    void *args[] = {&p, &last, &m, &final};
+    void *args[] = {&p, &last, &m, &turn, &final};
     return cudaLaunchKernelExC(&lc, fn, args);
 }
 
@@ -188,9 +188,11 @@ cudaError_t launch_tail(peel::Params<Off> &p, long long m, LastResult *last, cud
 // cluster kernel (which walks 5 M arcs at worst in 0.4 ms); large ones end with
 // the grid kernel. R-MAT scales 20 and 21 take 4.75 and 6.20 ms with six, 5.95
 // and 7.22 ms with four.
+constexpr int kMostLaunches = 12;
+static_assert(kMostLaunches < kMaxTurns, "every launch counts its CTAs in a word of its own");
 int tail_launches(long long m)
 {
-    return m < (6 << 20) ? 1 : m < (20 << 20) ? 3 : m < (120 << 20) ? 6 : 12;
+    return m < (6 << 20) ? 1 : m < (20 << 20) ? 3 : m < (120 << 20) ? 6 : kMostLaunches;
 }
 
 // Reads a range (16 bytes a thread per step); the values are not used.
@@ -276,9 +278,10 @@ int launch_turns(const peel::Params<Off> &p0, long long m, LastResult *last, cud
     const size_t win = std::min<size_t>((size_t)p.n * sizeof(int), cfg.l2_window);
     for (int i = 0; i < launches; ++i) {
         bool final = i + 1 == launches;
-        void *args[] = {&p, &last, &limit, &m, &final};
+        int turn = i + 1;
+        void *args[] = {&p, &last, &limit, &m, &turn, &final};
         const cudaError_t e =
-            i % 2 == 0 ? launch_tail(p, m, last, stream, cfg.device, final)
+            i % 2 == 0 ? launch_tail(p, m, last, stream, cfg.device, turn, final)
                        : launch_cooperative((const void *)peelone_kernel<Off, kPeelRepair, true, true>,
                                             dim3(ctas), dim3(kThreads), args, 0, stream, p.work, win);
         if (e != cudaSuccess) return -3;
@@ -347,7 +350,8 @@ int launch_peelone(const Off *rp, const int *ci, long long n, long long m, int *
     unsigned long long limit = cfg.limit_ns;
     const bool tail = async && mode == kPeelRepair;
     bool final = !tail;
-    void *args[] = {&p, &last, &limit, &m, &final};
+    int turn = 0;
+    void *args[] = {&p, &last, &limit, &m, &turn, &final};
     // the residual degrees (the target of every decrement) stay in L2
     const size_t win = async ? std::min<size_t>((size_t)n * sizeof(int), cfg.l2_window) : 0;
     if (launch_cooperative(fns[async][mode], grid, block, args, 0, stream, p.work, win) !=

@@ -99,7 +99,7 @@ enum PhaseKind : int {
 struct Ctrl {
     Line bar;                 // w[0..1]: arrivals at grid barriers (64-bit, whole launch)
     Line gen;                 // w[0]: grid barriers completed
-    Line stat;                // w[0] status, w[1] CTAs that finished
+    Line stat;                // w[0] status, w[1 + t] CTAs that finished launch t of the call
     Line live;                // counters updated with atomics
     Line snap[2];             // live counters as of the last barrier (by parity)
     Line tail;                // state shared by the launches of one PeelOne run (TailState)
@@ -343,15 +343,20 @@ __device__ __forceinline__ void fold_block(Ctrl *c, unsigned long long *st)
 // statistics into the call's control block; the last CTA publishes the
 // status and statistics to the per-device LastResult. True for the thread that
 // published them.
+// turn: the launch of the call, for calls of which several launches may finish
+// (their grids differ): each counts its own CTAs, so that a launch of which only some
+// finish, after a wait that ran out, does not keep a later one from publishing.
+constexpr int kMaxTurns = 31;
 __device__ __forceinline__ bool finish_block(Ctrl *c, LastResult *last, int algo,
-                                             const unsigned long long *local, int nlocal)
+                                             const unsigned long long *local, int nlocal,
+                                             int turn = 0)
 {
     __syncthreads();
     if (threadIdx.x == 0) {
         for (int i = 0; i < nlocal; ++i)
             if (local[i]) atomicAdd(&c->stats[i], local[i]);
         __threadfence();
-        unsigned done = atomicAdd(&c->stat.w[1], 1u);
+        unsigned done = atomicAdd(&c->stat.w[1 + turn], 1u);
         if (done == gridDim.x - 1) {
             __threadfence();
             int st = status_of(c);

@@ -87,3 +87,10 @@ def test_consecutive_waves(pico, make, off):
     for _ in range(3):
         launches, _ = peel(pico, g, off)
         assert launches >= 1
+
+
+def test_error_of_a_handed_over_call_is_reported(pico):
+    """A launch of which only some CTAs finish does not keep the narrower one
+    after it from publishing the error."""
+    assert pico.pico_selftest_handover() == pico.PICO_ERR_TIMEOUT
+    assert pico.pico_last_device_status() == pico.PICO_OK
