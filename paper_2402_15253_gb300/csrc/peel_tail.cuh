@@ -36,7 +36,9 @@
 //          Vertices that do not fit a queue are listed in global memory and
 //          walked with the next wave.
 //   bail   A wave of more than kTailBudget arcs goes back to the grid kernel,
-//          which finishes the level, unless this is the run's last launch.
+//          which finishes the level, unless this is the run's last launch. A
+//          wave of at most kTailThreads vertices is laid out by every CTA, which
+//          sees its arcs; those of a wider one are counted first (wave_arcs).
 // The run ends when every vertex is queued: the rest of the last level's walk
 // could only lower vertices that have their coreness.
 #pragma once
@@ -52,6 +54,16 @@ constexpr int kTailThreads = 512;
 constexpr int kTailQueue = 4096;         // queue entries of a CTA and wave
 constexpr int kTailNear = 8192;          // near-list entries of a CTA
 constexpr int kTailWindow = 32;          // first width of the near window
+
+// A row of d arcs in the sums that a wave is laid out by, which are 32 bits wide
+// (graphs have up to 2^36 arcs). Unless this is the run's last launch, a wave of more
+// than kTailBudget arcs goes back: one row of more is then counted as kTailBudget + 1,
+// and no sum over a tile's 512 rows wraps. The last launch of a run is one of
+// this kernel only for graphs of at most kTailMaxGraph arcs, where nothing wraps.
+__host__ __device__ inline int tail_row(long long d, bool last)
+{
+    return last || d <= (long long)kTailBudget ? (int)d : (int)kTailBudget + 1;
+}
 
 struct TailShared {
     long long off[kTailThreads];         // a wave's rows: row start minus position ...
@@ -274,7 +286,7 @@ struct TailPeel {
         int d = 0;
         if (v >= 0) {
             rs = p.rp[v];
-            d = (int)(p.rp[v + 1] - rs);
+            d = tail_row((long long)(p.rp[v + 1] - rs), last);
         }
         int incl = d;
 #pragma unroll
@@ -308,8 +320,31 @@ struct TailPeel {
         return true;
     }
 
+    // Arcs of a wave of more than kTailThreads vertices, each CTA's share counted as
+    // at most kTailBudget + 1 per warp (queue not walked yet: qb is the wave's buffer).
+    // Without it one CTA would walk a hub in such a wave alone: a wave of 600
+    // vertices, one of them with a million leaves, in a graph of 16.4 M arcs, 2.10 ms
+    // against 0.84 with it (R-MAT scale 22 and Chung-Lu 2^22 unchanged within 1 %).
+    __device__ __forceinline__ unsigned wave_arcs(const TailTotals &t, unsigned own)
+    {
+        unsigned sum = 0;
+        const auto add = [&](int v) {
+            sum += (unsigned)tail_row((long long)(p.rp[v + 1] - p.rp[v]), false);
+        };
+        // at most 8 own vertices a thread and 2^17 / 2^13 listed ones (queued * k is
+        // within the budget), so the sum of a warp does not wrap
+        for (unsigned i = threadIdx.x; i < own; i += blockDim.x) add(sh.queue[qb][i]);
+        for (unsigned i = rank * blockDim.x + threadIdx.x; i < t.queued - t.fitted;
+             i += (unsigned)kTailCtas * blockDim.x)
+            add(ldcg(p.fs + listed + i));
+        sum = min(__reduce_add_sync(kFull, sum), kTailBudget + 1);
+        if ((threadIdx.x & 31) == 0 && sum) atomicAdd(&sh.kept, sum);
+        return exchange(true).kept;
+    }
+
     // Walks the wave's vertices (buffer b). Returns false, with nothing walked,
-    // when they have more than the budget's arcs (decided alike by every CTA).
+    // when they have more than the budget's arcs (decided alike by every CTA); a wave
+    // of more than kTailThreads vertices was counted before.
     __device__ __forceinline__ bool wave(unsigned b, const TailTotals &t)
     {
         const unsigned total = t.queued;
@@ -323,7 +358,7 @@ struct TailPeel {
             int d = 0;
             if (v >= 0) {
                 rs = p.rp[v];
-                d = (int)(p.rp[v + 1] - rs);
+                d = tail_row((long long)(p.rp[v + 1] - rs), last);
             }
             int incl = d;
 #pragma unroll
@@ -486,7 +521,8 @@ struct TailPeel {
             while (t.queued > 0 && left > 0) {
                 const unsigned b = qb, own = min(sh.x[par ^ 1u][rank][0].x, (unsigned)kTailQueue);
                 settle(b, own);
-                if (!last && (unsigned long long)t.queued * (unsigned)k > kTailBudget) {
+                if (!last && ((unsigned long long)t.queued * (unsigned)k > kTailBudget ||
+                              (t.queued > T && wave_arcs(t, own) > kTailBudget))) {
                     mode = kTailPending;
                 } else {
                     qb ^= 1u;

@@ -192,7 +192,7 @@ constexpr int kMostLaunches = 12;
 static_assert(kMostLaunches < kMaxTurns, "every launch counts its CTAs in a word of its own");
 int tail_launches(long long m)
 {
-    return m < (6 << 20) ? 1 : m < (20 << 20) ? 3 : m < (120 << 20) ? 6 : kMostLaunches;
+    return m < (6 << 20) ? 1 : m < peel::kTailMaxGraph ? 3 : m < (120 << 20) ? 6 : kMostLaunches;
 }
 
 // Reads a range (16 bytes a thread per step); the values are not used.

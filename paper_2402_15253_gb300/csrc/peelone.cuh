@@ -92,6 +92,9 @@ struct TailState {
 constexpr unsigned kTailMaxResidual = 512u << 10;
 constexpr unsigned kTailMaxArcs = 64u << 10;
 constexpr unsigned kTailBudget = 128u << 10;
+// Largest graph whose run may end with a launch of the cluster kernel, which then
+// walks whatever is left.
+constexpr long long kTailMaxGraph = 20ll << 20;
 static_assert(sizeof(TailState) <= sizeof(Line), "the control block has no room for TailState");
 constexpr long long kTailSkew = 16;   // largest degree at least this many times the mean
 

@@ -94,3 +94,60 @@ def test_error_of_a_handed_over_call_is_reported(pico):
     after it from publishing the error."""
     assert pico.pico_selftest_handover() == pico.PICO_ERR_TIMEOUT
     assert pico.pico_last_device_status() == pico.PICO_OK
+
+
+def hub_in_wide_wave(core, leaves):
+    """A wave of 600 vertices at level 2, one of them with `leaves` neighbours that
+    left at level 1: more arcs than the cluster kernel may walk."""
+    a = core + torch.arange(300)
+    b = core + 300 + torch.arange(600)
+    leaf = core + 900 + torch.arange(leaves)
+    return union(core + 900 + leaves, circulant(core, 12), star(0, torch.arange(20, 8000)),
+                 (a.repeat_interleave(2), b), (b, torch.arange(600) * 7 + 1),
+                 (b, torch.arange(600) * 7 + 9001), star(int(b[77]), leaf))
+
+
+def five_tree(core):
+    """A tree of five children a vertex, whose 78,125 leaves hang on a dense part:
+    level 5 peels it from the root, and its last waves do not fit the queues."""
+    size = [5 ** i for i in range(8)]
+    first = [core + sum(size[:i]) for i in range(8)]
+    pairs = [circulant(core, 12), star(0, torch.arange(20, 6000))]
+    for i in range(1, 8):
+        ids = torch.arange(size[i])
+        pairs.append((first[i - 1] + ids // 5, first[i] + ids))
+    leaf = first[7] + torch.arange(size[7])
+    for j in range(5):
+        pairs.append((leaf, (torch.arange(size[7]) * 31 + j * 7001) % core))
+    return union(first[7] + size[7], *pairs)
+
+
+def alternating(parts):
+    """Heavy levels (9,000 vertices of a complete bipartite part each) with light
+    ones between them, next to a star."""
+    graphs = [gg.star_graph(90000)]
+    for i in range(parts):
+        k = 37 + 25 * i
+        left = torch.arange(k).repeat_interleave(9000)
+        graphs += [gg.csr_from_pairs(left, k + torch.arange(9000).repeat(k), k + 9000),
+                   gg.complete_graph(k + 6)]
+    return gg.disjoint_union(graphs)
+
+
+TURNS = [
+    # (graph, launches that peel on the cluster, waves the grid kernel takes back)
+    ("wide-wave-with-hub", lambda: hub_in_wide_wave(300000, 200000), None, 1),
+    ("wide-wave-with-hub-last", lambda: hub_in_wide_wave(70000, 200000), 1, 0),
+    ("spilled-last", lambda: five_tree(60000), 1, 0),
+    ("spilled-back", lambda: five_tree(300000), None, 1),
+    ("turns-end-on-the-cluster", lambda: alternating(7), 2, 1),
+    ("turns-end-on-the-grid", lambda: alternating(10), 3, 3),
+]
+
+
+@pytest.mark.parametrize("off", [torch.int32, torch.int64], ids=["int32", "int64"])
+@pytest.mark.parametrize("name,make,clusters,back", TURNS, ids=[t[0] for t in TURNS])
+def test_turns(pico, name, make, clusters, back, off):
+    launches, taken_back = peel(pico, make(), off)
+    assert launches == clusters if clusters is not None else launches >= 1
+    assert taken_back >= back if clusters is None else taken_back == back
