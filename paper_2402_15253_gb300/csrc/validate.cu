@@ -48,6 +48,21 @@ __global__ void __launch_bounds__(256)
 
 constexpr int kSegment = 512;   // most arcs of a warp's turn in the quick pass
 
+// The last row in [lo, hi) that starts at or before arc a, by 32-way search (one
+// warp); rp[lo] <= a < rp[hi].
+template <typename Off>
+__device__ __forceinline__ long long row_at(const Off *rp, long long lo, long long hi, long long a)
+{
+    const int lane = threadIdx.x & 31;
+    while (hi - lo > 1) {
+        const long long step = (hi - lo + 31) / 32, at = lo + (lane + 1) * step;
+        const unsigned b = __ballot_sync(kFull, at < hi && (long long)rp[at] <= a);
+        lo += (long long)__popc(b) * step;   // the probes that pass come first
+        hi = lo + step < hi ? lo + step : hi;
+    }
+    return lo;
+}
+
 // segment: arcs of a warp's turn, a multiple of 32
 template <typename Off>
 __global__ void __launch_bounds__(256)
@@ -65,14 +80,7 @@ __global__ void __launch_bounds__(256)
     for (long long seg = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; seg < nseg;
          seg += nw) {
         const long long a0 = seg * segment, a1 = a0 + segment < m ? a0 + segment : m;
-        // the last row that starts at or before a0, by 32-way search: rp[lo] <= a0 < rp[hi]
-        long long lo = 0, hi = n;
-        while (hi - lo > 1) {
-            const long long step = (hi - lo + 31) / 32, at = lo + (lane + 1) * step;
-            const unsigned b = __ballot_sync(kFull, at < hi && (long long)rp[at] <= a0);
-            lo += (long long)__popc(b) * step;   // the probes that pass come first
-            hi = lo + step < hi ? lo + step : hi;
-        }
+        long long lo = row_at(rp, 0, n, a0);
         for (long long w = a0; w < a1; w += 32) {
             const long long e = w + lane;
             // the row of each arc: the starts of the next 32 rows, and again
@@ -89,8 +97,15 @@ __global__ void __launch_bounds__(256)
                     if (__shfl_sync(kFull, start, c + s - 1) <= mine) c += s;
                 if (__shfl_sync(kFull, start, c) <= mine) ++c;   // c <= 31 here
                 if (c > 0) v = lo + c;
-                if (__shfl_sync(kFull, start, 31) > last) break;
+                const long long end = __shfl_sync(kFull, start, 31);
+                if (end > last) break;
                 lo += 32;
+                if (__shfl_sync(kFull, start, 0) == end) {
+                    // a run of empty rows, which may be millions of rows long (ids
+                    // that are not used): its end is searched for
+                    lo = row_at(rp, lo, n, end);
+                    if (c > 0) v = lo;
+                }
             }
             lo = __shfl_sync(kFull, v, 31);
             if (e >= a1) continue;

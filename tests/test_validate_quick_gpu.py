@@ -1,6 +1,8 @@
 """Validation of a graph in even shares of its arcs: rows that begin and end
 around a share (512 arcs), runs of empty rows, hubs, and single defects
 anywhere must be judged as by a plain check of every arc."""
+import time
+
 import numpy as np
 import pytest
 import torch
@@ -82,3 +84,35 @@ def test_shares_of_arcs(pico, name, make, off):
             else:
                 assert bits == want, (at, value)
             assert (status == pico.PICO_OK) == (bits == 0)
+
+
+@pytest.mark.parametrize("off", [torch.int32, torch.int64], ids=["int32", "int64"])
+@pytest.mark.parametrize("gap", [31, 32, 33, 63, 64, 65, 95, 96, 97, 1023, 1024, 1025, 1 << 20])
+def test_runs_of_empty_rows(pico, gap, off):
+    """Used ids with runs of unused ones between them, inside one share of arcs."""
+    g = spread([gg.complete_graph(3), gg.path_graph(2), gg.complete_graph(4)] * 2, gap)
+    rp, ci = g.numpy()
+    check = pico.pico_validate_graph if off == torch.int32 else pico.pico_validate_graph_i64
+    drp = torch.from_numpy(rp).to("cuda", dtype=off)
+    assert check(drp, torch.from_numpy(ci).cuda(), g.n, len(ci)) == (pico.PICO_OK, 0)
+    for at in range(len(ci)):
+        bad = ci.copy()
+        bad[at] = ci[at - 1]
+        want = defects(pico, rp, bad)
+        status, bits = check(drp, torch.from_numpy(bad).cuda(), g.n, len(ci))
+        assert bits & ~pico.PICO_DEFECT_ASYMMETRIC == want & ~pico.PICO_DEFECT_ASYMMETRIC, at
+        assert (status == pico.PICO_OK) == (want == 0), at
+
+
+def test_long_run_of_empty_rows_is_not_walked(pico):
+    """2^23 unused ids between two used ranges: some 20 dependent steps, not a
+    quarter of a million (95 ms)."""
+    g = spread([gg.complete_graph(5)] * 2, 1 << 23)
+    rp, ci = g.row_ptr.cuda(), g.col_idx.cuda()
+    times = []
+    for _ in range(4):
+        torch.cuda.synchronize()
+        t0 = time.perf_counter()
+        assert pico.pico_validate_graph(rp, ci, g.n, g.arcs) == (pico.PICO_OK, 0)
+        times.append(time.perf_counter() - t0)
+    assert min(times) < 0.02
