@@ -195,12 +195,14 @@ int launch_validate(const Off *rp, const int *ci, long long n, long long m, Vali
     const int segment =
         (int)std::min<long long>(kSegment, std::max<long long>(32, (m / (8 * most) + 31) & ~31ll));
     const unsigned blocks = (unsigned)std::min<long long>(most, n / 256 + 1);
+    // the exact kernel takes a warp for every row, if it has anything to do
+    const unsigned exact = (unsigned)std::min<long long>(most, n / 8 + 1);
     const unsigned shares = (unsigned)std::min<long long>(most, m / (8 * segment) + 1);
     validate_rows<Off><<<blocks, 256, 0, stream>>>(rp, n, m, &words->defects);
     if (cudaGetLastError() != cudaSuccess) return -3;
     validate_quick<Off><<<shares, 256, 0, stream>>>(rp, ci, n, m, segment, words);
     if (cudaGetLastError() != cudaSuccess) return -3;
-    validate_arcs<Off><<<blocks, 256, 0, stream>>>(rp, ci, n, words);
+    validate_arcs<Off><<<exact, 256, 0, stream>>>(rp, ci, n, words);
     if (cudaGetLastError() != cudaSuccess) return -3;
     return 0;
 }

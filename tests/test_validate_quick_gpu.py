@@ -116,3 +116,19 @@ def test_long_run_of_empty_rows_is_not_walked(pico):
         assert pico.pico_validate_graph(rp, ci, g.n, g.arcs) == (pico.PICO_OK, 0)
         times.append(time.perf_counter() - t0)
     assert min(times) < 0.02
+
+
+def test_malformed_graph_costs_little_more(pico):
+    """One bad id among 2,000 rows of 200 arcs: the exact kernel that names the
+    defect has a warp for every row (a 32nd of them took seven times as long)."""
+    g = gg.er_graph(2000, 200000, 9)
+    rp, ci = g.row_ptr.cuda(), g.col_idx.cuda()
+    bad = ci.clone()
+    bad[g.arcs // 2] = g.n
+    best = {}
+    for name, c, want in (("valid", ci, 0), ("bad", bad, pico.PICO_DEFECT_IDS)) * 8:
+        torch.cuda.synchronize()
+        t0 = time.perf_counter()
+        assert pico.pico_validate_graph(rp, c, g.n, g.arcs)[1] & want == want
+        best[name] = min(best.get(name, 1.0), time.perf_counter() - t0)
+    assert best["bad"] < 3 * best["valid"]
