@@ -68,13 +68,18 @@
 // Compacted chunks. A pushed edit reaches u only when K = core[u] is above y,
 // and the neighbours of a hub mostly lie far below: on a Chung-Lu graph of 2^24
 // vertices a round that changes 2,000 hubs gathers 50 M records to edit 1 % of
-// them, at the rate L2 serves them. So the first push of a chunk writes the
-// neighbours with K > y / 2 to the chunk's place in an array like col_idx
-// (`near`: their number, the bound y / 2, the neighbours). Estimates only fall,
-// so while y stays at or above the bound the others cannot be above y either,
-// and later pushes walk that list; below the bound it is built again. A chunk
-// most of whose neighbours qualify is left alone. Replayed on R-MAT scale 18 and
-// Chung-Lu 2^18, half and an eighth of the pushed arcs remain.
+// them, at the rate L2 serves them. So the first push of a chunk lists the
+// neighbours with K > y / 2, and later pushes walk that list: estimates only fall,
+// so while y stays at or above the bound y / 2 the others cannot be above y
+// either. Below the bound the list is built again. A chunk most of whose neighbours
+// qualify is left alone. Replayed on R-MAT scale 18 and Chung-Lu 2^18, half and an
+// eighth of the pushed arcs remain.
+// The lists need no memory of their own: the slots of a histogram row above the
+// vertex's estimate are never read or edited again, and a hub's estimate is far
+// below its degree. A chunk keeps its list at the end of its own slots, as far as
+// they lie above the estimate when the list is built. Chung-Lu 2^24: 27.0 ms without
+// lists, 21.0 with them in m ints of their own, 21.0 in the rows; R-MAT scale 24: 53.0,
+// 52.6, 52.1 ms.
 //
 // Load balance. V_cnt is kept as three lists by the estimate K that SumHisto
 // will walk down from: K <= 32 one thread per vertex, K <= 2048 one warp per
@@ -147,13 +152,16 @@ struct Params {
     // rounded up to 4; zero between rounds); nullptr: pull rounds decide the
     // append at the edit, as push rounds do.
     unsigned char *cand = nullptr;
-    // Compacted chunks (m ints; nullptr: pushes walk every arc). The chunk that
-    // starts at arc s, if it has at least kNearMin arcs: near[s] is the number
-    // of neighbours listed from near[s + 2] on, or kNearNone (not built) or
-    // kNearFull (not worth it); near[s + 1] the bound.
-    int *near = nullptr;
+    // Compacted chunks: lists in the histogram rows (see above); false: pushes walk
+    // every arc. The last two slots of a chunk are kListMark | room << 14 | the
+    // number of neighbours listed in the `room` slots before them (kListFull: not
+    // worth a list), and the bound. A count that a slot was left with is never a
+    // mark: its two top bits are equal.
+    bool lists = false;
 };
-constexpr int kNearMin = 16, kNearNone = -1, kNearFull = -2;
+constexpr int kListMin = 16;   // fewest slots above the estimate that are used
+constexpr unsigned kListMark = 0x80000000u, kListTop = 0xc0000000u, kListFull = 0x3fffu;
+static_assert(kMaxChunk < (int)kListFull, "a list's room and number have 14 bits each");
 
 // Packed {old, new} record: old << 16 | new when old <= 65534 (new < old);
 // kMvpWide otherwise (never a packed value, since new < old).
@@ -288,7 +296,7 @@ struct UpdateArc {
 };
 
 // One warp pushes chunk c of changed vertex v, from its compacted list when
-// there is one for the vertex's new estimate (see Params::near).
+// there is one for the vertex's new estimate (see Params::lists).
 template <typename Off>
 __device__ __forceinline__ void push_chunk(const Params<Off> &p, int v, int c, UpdateArc<Off> &f)
 {
@@ -301,21 +309,26 @@ __device__ __forceinline__ void push_chunk(const Params<Off> &p, int v, int c, U
     f.item(v, x, y);
     const int *arcs = p.ci + s;
     bool build = false, compacted = false;
-    if (p.near && len >= kNearMin) {
-        int *head = p.near + s;
-        const int h = ldcg(head + (lane & 1));   // lane 0: the number, lane 1: the bound
-        const int number = __shfl_sync(kFull, h, 0), bound = __shfl_sync(kFull, h, 1);
-        if (number != kNearNone && y >= bound) {
-            if (number >= 0) {
-                arcs = head + 2;
-                len = number;
+    int *const head = p.histo + s + len - 2;
+    // slots of the chunk above the estimate: len in all, those up to y are in use
+    const long long above = (long long)c * p.tn.chunk + len - y;
+    const int dead = above < len ? (int)above : len;
+    if (p.lists && dead >= kListMin) {
+        const int h = ldcg(head + (lane & 1));   // lane 0: the mark, lane 1: the bound
+        const unsigned mark = (unsigned)__shfl_sync(kFull, h, 0);
+        const int bound = __shfl_sync(kFull, h, 1);
+        if ((mark & kListTop) == kListMark && y >= bound) {
+            const unsigned number = mark & kListFull;
+            if (number != kListFull) {
+                arcs = head - ((mark >> 14) & kListFull);
+                len = (int)number;
                 compacted = true;
             }
         } else {
             build = true;
-            f.list = head + 2;
             f.bound = y >> 1;
-            f.room = len - len / 4 - 2;   // the list and its head fit the chunk
+            f.room = min(len - len / 4, dead) - 2;
+            f.list = head - f.room;
             f.listed = 0;
         }
     }
@@ -338,8 +351,9 @@ __device__ __forceinline__ void push_chunk(const Params<Off> &p, int v, int c, U
     }
     if (build) {
         if (lane == 0) {
-            p.near[s] = f.listed <= f.room ? f.listed : kNearFull;
-            p.near[s + 1] = f.bound;
+            head[0] = (int)(kListMark | (unsigned)f.room << 14 |
+                            (f.listed <= f.room ? (unsigned)f.listed : kListFull));
+            head[1] = f.bound;
         }
         f.list = nullptr;
     }
@@ -724,11 +738,6 @@ __device__ void run(const Params<Off> &p0, Dom &dom, unsigned *s_tmp, unsigned l
     // InitHisto
     {
         InitArc<Off> f{p.vinfo, p.histo};
-        if (p.near)   // no chunk is compacted yet
-            for (unsigned i = tid; i < nib; i += nthreads) {
-                const int2 e = __ldcg(ilist + i);
-                p.near[p.rp[e.x] + (Off)e.y * p.tn.chunk] = kNearNone;
-            }
         expand(p.rp, p.ci, (const int *)nullptr, (unsigned)n, ilist, nib, gwarp, nwarps, f, p.tn);
         arcs += f.n_arcs;
         atomics += f.n_arcs;

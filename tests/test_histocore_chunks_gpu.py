@@ -64,3 +64,38 @@ def test_rounds_match_oracle(pico, name, make, off, mode):
     assert st["slots"] == ost["slots_read"]
     assert st["arcs"] == g.arcs + ost["arcs_scanned"]
     assert st["atomics"] == g.arcs + 2 * ost["updates"]
+
+
+def rings_of_hubs(hubs, deg, step):
+    """Hubs of `deg` to `deg + step * hubs` neighbours each, joined to each other:
+    chunks of which none, a few or all slots lie above the hub's estimate."""
+    i, j = torch.triu_indices(hubs, hubs, 1)
+    s, d, at = [i], [j], hubs
+    for h in range(hubs):
+        k = deg + step * h
+        leaf = at + torch.arange(k)
+        s += [torch.full((k,), h), leaf[:-1], leaf[:-2]]
+        d += [leaf, leaf[1:], leaf[2:]]
+        at += k
+    return gg.csr_from_pairs(torch.cat(s), torch.cat(d), at)
+
+
+@pytest.mark.parametrize("chunk", [64, 256, 4096])
+@pytest.mark.parametrize("deg,step", [(1, 1), (190, 3), (460, 7)], ids=str)
+def test_lists_within_the_rows(pico, chunk, deg, step):
+    """Every chunk size: lists at the end of chunks that are partly in use."""
+    g = rings_of_hubs(60, deg, step)
+    rp, ci = g.numpy()
+    assert pico.pico_set_histo_update(pico.PICO_UPDATE_PUSH, 50) == 0
+    assert pico.pico_set_tuning(32, chunk, 512, 21) == 0
+    try:
+        for off in (torch.int32, torch.int64):
+            got = pico.coreness(g.row_ptr.to("cuda", dtype=off), g.col_idx.cuda(), "histocore")
+            st = pico.pico_get_stats()
+            assert np.array_equal(got.cpu().numpy(), oracle.bz_coreness(rp, ci))
+            _, ost = oracle.histocore(rp, ci)
+            assert st["rounds"] == ost["rounds"] and st["frontier"] == ost["frontier"]
+            assert st["slots"] == ost["slots_read"]
+            assert st["atomics"] == g.arcs + 2 * ost["updates"]
+    finally:
+        pico.pico_set_tuning(32, 256, 512, 21)
