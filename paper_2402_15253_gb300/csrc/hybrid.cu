@@ -38,7 +38,7 @@ __device__ __forceinline__ bool prefer_histocore(long long n, long long m, unsig
 template <typename Off>
 __global__ void __launch_bounds__(kThreads, 2)
     hybrid_kernel(peel::Params<Off> pp, histo::Params<Off> hp, LastResult *last,
-                  unsigned long long limit_ns, bool local)
+                  unsigned long long limit_ns, bool local, bool any_degrees)
 {
     __shared__ unsigned s_snap[kLiveWords + 1];
     __shared__ unsigned s_tmp[256];
@@ -68,11 +68,11 @@ __global__ void __launch_bounds__(kThreads, 2)
         use_histo = prefer_histocore(n, hp.m, s_snap[kLiveDmax]);
         if (use_histo)
             histo::run(hp, dom, s_tmp, st, clk, arcs, atomics, slots, pulled);
-        else if (local)
+        else if (local && (any_degrees || peel::local_degrees(s_snap[kLiveDmax], n, hp.m)))
             over = false;   // the next launch peels the graph in shared memory
         else if (pp.work)
             over = peel::run_async<Off, kPeelRepair, true>(pp, dom, s_tmp, st, clk, arcs, atomics,
-                                                           extra, false);
+                                                           extra, local);
         else
             peel::run<Off, GridDom, kPeelRepair>(pp, dom, s_tmp, st, clk, arcs, atomics, extra);
     }
@@ -158,8 +158,8 @@ int launch_hybrid(const Off *rp, const int *ci, long long n, long long m, int *c
     }
     if (cudaMemsetAsync(pp.ctl, 0, sizeof(Ctrl), stream) != cudaSuccess) return -3;
     unsigned long long limit = cfg.limit_ns;
-    bool local = pp.work && peelone_local(n, m);
-    void *args[] = {&pp, &hp, &last, &limit, &local};
+    bool local = pp.work && peelone_local(n, m, false), any_degrees = peelone_local(n, m, true);
+    void *args[] = {&pp, &hp, &last, &limit, &local, &any_degrees};
     // PeelOne's residual degrees stay in L2 (when HistoCore runs, the window
     // covers part of its scratch instead, which is harmless)
     const size_t win = pp.work ? std::min<size_t>((size_t)n * sizeof(int), cfg.l2_window) : 0;

@@ -28,6 +28,14 @@ constexpr int kLocalThreads = 1024;
 // 0.43 M: 545 against 1,503 us; Chung-Lu, n 32,768, m 0.6 M: 794 against 1,229
 // us with the cluster kernel and 2,028 us without).
 constexpr long long kLocalMaxArcs = 640 << 10;
+// Up to here whatever the degrees; beyond it a graph without skew has waves wide
+// enough for the grid, which then looks at the degrees first and keeps such a graph
+// (Erdos-Renyi, one CTA against the grid: n 10,000, mean degree 8: 166 and 218 us, 40:
+// 329 and 338 us; n 15,000: 190 and 222, 386 and 361 us; n 20,000, degree 8: 220 and
+// 226 us; 30,000: 292 and 234; 51,000: 438 and 228 us. With skew, R-MAT of 51,000
+// vertices: 814 and 1,317 us; grids of 51,000 vertices: 888 and 1,083 us).
+constexpr long long kLocalAnyVertices = 20480, kLocalAnyArcs = 400 << 10;   // both, ...
+constexpr long long kLocalFewVertices = 12288;                              // ... or this few
 
 // kTail: one of the launches that alternate with the cluster kernel. The one
 // that ends the run publishes the status and the statistics (the `final` one
@@ -35,7 +43,7 @@ constexpr long long kLocalMaxArcs = 640 << 10;
 template <typename Off, int Mode, bool kAsync, bool kTail>
 __global__ void __launch_bounds__(kThreads, 2)
     peelone_kernel(peel::Params<Off> p, LastResult *last, unsigned long long limit_ns,
-                   long long m, int turn, bool final)
+                   long long m, int turn, bool final, bool local)
 {
     __shared__ unsigned s_snap[kLiveWords + 1];
     __shared__ unsigned s_tmp[128];
@@ -55,7 +63,8 @@ __global__ void __launch_bounds__(kThreads, 2)
     GridDom dom{p.ctl, s_snap, limit_ns};
     bool over = true;
     if (kAsync)
-        over = peel::run_async<Off, Mode, kTail>(p, dom, s_tmp, st, clk, arcs, atomics, extra, final);
+        over = peel::run_async<Off, Mode, kTail>(p, dom, s_tmp, st, clk, arcs, atomics, extra, final,
+                                                 local);
     else
         peel::run<Off, GridDom, Mode>(p, dom, s_tmp, st, clk, arcs, atomics, extra);
     if (kTail) {   // every row is expanded once, by one kernel or the other
@@ -242,9 +251,10 @@ size_t peelone_ws_bytes(long long n, long long m, bool async)
     return c.size();
 }
 
-bool peelone_local(long long n, long long m)
+bool peelone_local(long long n, long long m, bool any_degrees)
 {
-    return n <= peel::kLocalSlots && m <= kLocalMaxArcs;
+    if (n > peel::kLocalSlots || m > kLocalMaxArcs) return false;
+    return !any_degrees || n <= kLocalFewVertices || (n <= kLocalAnyVertices && m <= kLocalAnyArcs);
 }
 
 template <typename Off>
@@ -279,7 +289,8 @@ int launch_turns(const peel::Params<Off> &p0, long long m, LastResult *last, cud
     for (int i = 0; i < launches; ++i) {
         bool final = i + 1 == launches;
         int turn = i + 1;
-        void *args[] = {&p, &last, &limit, &m, &turn, &final};
+        bool local = false;
+        void *args[] = {&p, &last, &limit, &m, &turn, &final, &local};
         const cudaError_t e =
             i % 2 == 0 ? launch_tail(p, m, last, stream, cfg.device, turn, final)
                        : launch_cooperative((const void *)peelone_kernel<Off, kPeelRepair, true, true>,
@@ -312,7 +323,7 @@ int launch_peelone(const Off *rp, const int *ci, long long n, long long m, int *
                               (const void *)peelone_kernel<Off, kPeelAddBack, true, false>}};
     static int occ[2][3][64] = {};
     bool async = cfg.peel_async;
-    if (async && mode == kPeelRepair && peelone_local(n, m)) {
+    if (async && mode == kPeelRepair && peelone_local(n, m, true)) {
         Carver c(ws);
         peel::Params<Off> p;
         peel::carve(p, c, n, m, true);
@@ -349,15 +360,18 @@ int launch_peelone(const Off *rp, const int *ci, long long n, long long m, int *
     dim3 grid(ctas), block(kThreads);
     unsigned long long limit = cfg.limit_ns;
     const bool tail = async && mode == kPeelRepair;
-    bool final = !tail;
+    bool local = tail && peelone_local(n, m, false);   // this launch or one CTA, by the degrees
+    bool final = !tail || local;
     int turn = 0;
-    void *args[] = {&p, &last, &limit, &m, &turn, &final};
+    void *args[] = {&p, &last, &limit, &m, &turn, &final, &local};
     // the residual degrees (the target of every decrement) stay in L2
     const size_t win = async ? std::min<size_t>((size_t)n * sizeof(int), cfg.l2_window) : 0;
     if (launch_cooperative(fns[async][mode], grid, block, args, 0, stream, p.work, win) !=
         cudaSuccess)
         return -3;
-    if (tail && launch_turns(p, m, last, stream, cfg, ctas) != 0) return -3;
+    if (tail && (local ? launch_local(p, m, p.tail, last, stream, cfg)
+                       : launch_turns(p, m, last, stream, cfg, ctas)) != 0)
+        return -3;
     if (win > 0 && l2_release(p.work, win, stream) != cudaSuccess) return -3;
     return 0;
 }

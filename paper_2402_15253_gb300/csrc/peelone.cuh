@@ -98,6 +98,15 @@ constexpr long long kTailMaxGraph = 20ll << 20;
 static_assert(sizeof(TailState) <= sizeof(Line), "the control block has no room for TailState");
 constexpr long long kTailSkew = 16;   // largest degree at least this many times the mean
 
+// Whether a graph of the size for it (peelone_local) is better peeled by one CTA in
+// shared memory, if that hangs on its degrees (see kLocalAnyVertices): skewed ones
+// and lattices have many levels or waves of few arcs.
+constexpr unsigned kLocalLattice = 8;   // largest degree of a lattice
+__host__ __device__ inline bool local_degrees(unsigned dmax, long long n, long long m)
+{
+    return dmax <= kLocalLattice || (long long)dmax * n >= kTailSkew * m;
+}
+
 template <typename Off>
 struct Params {
     const Off *rp;
@@ -617,7 +626,8 @@ __device__ __forceinline__ void walk_chunk_guarded(const Off *__restrict__ rp,
 template <typename Off, int Mode = kPeelRepair, bool kTail = false>
 __device__ bool run_async(const Params<Off> &p, GridDom &dom, unsigned *s_tmp,
                           unsigned long long *st, PhaseClock &clk, unsigned long long &arcs,
-                          unsigned long long &atomics, unsigned long long &extra, bool last = true)
+                          unsigned long long &atomics, unsigned long long &extra, bool last = true,
+                          bool local = false)
 {
     Ctrl *ctl = p.ctl;
     unsigned *live = dom.live();
@@ -688,6 +698,7 @@ __device__ bool run_async(const Params<Off> &p, GridDom &dom, unsigned *s_tmp,
         nres = snap[L_KEPT];
         k = INT_MAX - (int)snap[L_MIN];
         if (kTail) skewed = (long long)snap[L_DMAX] * n >= kTailSkew * (long long)p.rp[n];
+        if (kTail && local && local_degrees(snap[L_DMAX], n, (long long)p.rp[n])) return false;
     } else {
         nres = p.tail->nres;
         k = p.tail->k;

@@ -99,8 +99,9 @@ struct TailState;
 }  // namespace peel
 
 // Whether a graph of this size is peeled in one CTA's shared memory
-// (launch_local) instead of by the grid kernel.
-bool peelone_local(long long n, long long m);
+// (launch_local) instead of by the grid kernel: whatever its degrees, or if they call
+// for it (peel::local_degrees, known on the device).
+bool peelone_local(long long n, long long m, bool any_degrees);
 
 // The shared-memory form; p: carved scratch with the control block zeroed.
 // tail: the launch does nothing when *tail says the call is published.
