@@ -245,8 +245,12 @@ __device__ __forceinline__ peel::LocalParams<int> local_params(const BatchParams
 // PeelOne, huge graphs: one cluster per graph. Bound by the latency of L2 atomics
 // and of the cluster barriers; 8 CTAs of 512 threads, two to an SM, keep twice the
 // warps that 4 CTAs of 1,024 have, and leave room for a second graph beside them
-// (one R-MAT graph of 2^20 vertices and 31 M arcs: 35 -> 16.5 ms; 24 of them and
-// 488 smaller graphs: 41.8 -> 23.7 ms).
+// (one R-MAT graph of 2^20 vertices and 31 M arcs: 35 ms with those, 15.9 ms so; 24 of them
+// and 488 smaller graphs: 41.8 and 24.4 ms).
+// Its reads of residual degrees hit in L1, so it prefers all of an SM's memory as L1.
+// Without that preference it starts on the SMs that another stream's wide CTAs
+// have left with 28 KB of L1, and takes 43 ms instead of 21 (two or four streams of
+// such batches: 35.7 ms a batch, 22.4 with it, 25.4 with one kernel for all classes).
 __global__ void __launch_bounds__(512, 2) batched_huge_kernel(BatchParams bp)
 {
     namespace cg = cooperative_groups;
@@ -365,10 +369,11 @@ __global__ void __launch_bounds__(kTinyThreads, 8) batched_tiny_kernel(BatchPara
 // Launches a kernel over a persistent grid of clusters: every cluster that is
 // resident at once, but no more than `need`. occ: the kernel's cached number
 // of resident clusters (0: not known yet). beside: the launch may run beside the
-// one before it on the stream.
+// one before it on the stream. carveout: percent of an SM's shared memory the kernel
+// prefers (-1: no preference).
 cudaError_t launch_clusters(const void *fn, int cluster, int threads, size_t smem, int sms,
                             long long need, int &occ, void **args, cudaStream_t stream,
-                            bool beside = false)
+                            bool beside = false, int carveout = -1)
 {
     cudaLaunchConfig_t lc = {};
     cudaLaunchAttribute attr[2];
@@ -385,6 +390,11 @@ cudaError_t launch_clusters(const void *fn, int cluster, int threads, size_t sme
         if (smem > 0) {
             const cudaError_t e =
                 cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+        }
+        if (carveout >= 0) {
+            const cudaError_t e =
+                cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, carveout);
             if (e != cudaSuccess) return e;
         }
         lc.gridDim = dim3(cluster * sms);
@@ -465,7 +475,8 @@ int launch_batched(const int64_t *vtx_off, const int64_t *arc_off, int G, const 
         const long long huge =
             std::min<long long>(G, total_n / ((long long)kPeelCtas * peel::kLocalSlots + 1));
         if (huge > 0 && launch_clusters((const void *)batched_huge_kernel, kClusterCtas, 512, 0,
-                                        cfg.sms, huge, occ_huge[dev], args, stream) != cudaSuccess)
+                                        cfg.sms, huge, occ_huge[dev], args, stream, false,
+                                        cudaSharedmemCarveoutMaxL1) != cudaSuccess)
             return -3;
         const long long wide = std::min<long long>(G, total_n / (kTinyVertices + 1));
         if (wide > 0 &&
