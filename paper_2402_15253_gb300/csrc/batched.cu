@@ -9,7 +9,8 @@
 // PeelOne keeps the residual degrees in shared memory (peel_local.cuh):
 //   tiny    n <= kTinyVertices: CTAs of kTinyThreads threads, eight per SM, so
 //           that one graph's barriers and chains overlap the others'.
-//   middle  n <= kLocalSlots: one CTA of kWideThreads threads per graph.
+//   middle  n <= kLocalSlots: one CTA of kWideThreads threads per graph; and tiny
+//           graphs that the rest of the batch would wait for (straggles).
 //   large   n <= kPeelCtas * kLocalSlots: a cluster of kPeelCtas CTAs per graph.
 //   huge    the rest: a cluster of kClusterCtas CTAs per graph, in global memory
 //           (peel::run over the cluster).
@@ -72,14 +73,27 @@ __device__ __forceinline__ int size_bucket(long long m)
     return m <= 0 ? 0 : 64 - __clzll(m);
 }
 
+// Whether a tiny graph takes a whole SM all the same: it has more arcs than an SM's
+// share of the batch (`share`), so its 128 threads would be the last at work. Graphs of
+// 2,000 vertices and 0.72 M arcs, Erdos-Renyi: 64 of them 1,432 us as tiny ones, 384 as
+// middle ones (1,213 with 512 threads for each); 512 of them 1,468 and 1,233; with 0.2 M
+// arcs 64 take 399 and 190 us, 512 take 423 and 510. Smaller graphs stay tiny: they take
+// less time than with 512 threads each in any batch.
+constexpr long long kTinyArcs = 32 << 10;
+__device__ __forceinline__ bool straggles(long long m, long long share)
+{
+    return m > kTinyArcs && m > share;
+}
+
 // Class of a graph: 3 (listed first) to 0. PeelOne: by where its residual
 // degrees fit; HistoCore: by its arcs (classes 2 and 0).
-__device__ __forceinline__ int graph_class(long long n, long long m, int algo, int cluster_log2)
+__device__ __forceinline__ int graph_class(long long n, long long m, int algo, int cluster_log2,
+                                           long long share)
 {
     if (algo != 0) return size_bucket(m) > cluster_log2 ? 2 : 0;
     return n > (long long)kPeelCtas * peel::kLocalSlots ? 3
            : n > peel::kLocalSlots                      ? 2
-                                                        : (n > kTinyVertices ? 1 : 0);
+                                                        : (n > kTinyVertices || straggles(m, share) ? 1 : 0);
 }
 
 // Lists the graphs by class and decreasing arc-count bucket (one CTA) and
@@ -87,7 +101,7 @@ __device__ __forceinline__ int graph_class(long long n, long long m, int algo, i
 // in [2^(b-1), 2^b)).
 __global__ void __launch_bounds__(1024)
     schedule_kernel(const long long *vtx_off, const long long *arc_off, int G, int *order, Ctrl *ctl,
-                    int algo, int cluster_log2)
+                    int algo, int cluster_log2, long long share)
 {
     __shared__ unsigned cnt[4 * kBuckets];
     __shared__ unsigned start[4 * kBuckets];
@@ -95,7 +109,7 @@ __global__ void __launch_bounds__(1024)
     __syncthreads();
     auto key = [&](int g) {
         const long long n = vtx_off[g + 1] - vtx_off[g], m = arc_off[g + 1] - arc_off[g];
-        return graph_class(n, m, algo, cluster_log2) * kBuckets + size_bucket(m);
+        return graph_class(n, m, algo, cluster_log2, share) * kBuckets + size_bucket(m);
     };
     for (int g = threadIdx.x; g < G; g += blockDim.x) atomicAdd(&cnt[key(g)], 1u);
     __syncthreads();
@@ -289,7 +303,7 @@ __global__ void __launch_bounds__(512, 2) batched_huge_kernel(BatchParams bp)
     cluster.sync();   // no CTA leaves while another may still read its shared memory
 }
 
-// PeelOne, large and middle graphs.
+// PeelOne, large and middle graphs (and tiny ones that straggle).
 __global__ void __launch_bounds__(kWideThreads, 1) batched_peel_kernel(BatchParams bp)
 {
     namespace cg = cooperative_groups;
@@ -464,7 +478,7 @@ int launch_batched(const int64_t *vtx_off, const int64_t *arc_off, int G, const 
     bp.tn = cfg.tn;
     if (cudaMemsetAsync(bp.ctl, 0, sizeof(Ctrl), stream) != cudaSuccess) return -3;
     schedule_kernel<<<1, 1024, 0, stream>>>(bp.vtx_off, bp.arc_off, G, bp.order, bp.ctl, algo,
-                                            cfg.tn.cluster_log2);
+                                            cfg.tn.cluster_log2, total_m / std::max(1, cfg.sms));
     if (cudaGetLastError() != cudaSuccess) return -3;
 
     const int dev = cfg.device & 63;
@@ -478,7 +492,8 @@ int launch_batched(const int64_t *vtx_off, const int64_t *arc_off, int G, const 
                                         cfg.sms, huge, occ_huge[dev], args, stream, false,
                                         cudaSharedmemCarveoutMaxL1) != cudaSuccess)
             return -3;
-        const long long wide = std::min<long long>(G, total_n / (kTinyVertices + 1));
+        const long long wide =
+            std::min<long long>(G, total_n / (kTinyVertices + 1) + total_m / (kTinyArcs + 1));
         if (wide > 0 &&
             launch_clusters((const void *)batched_peel_kernel, kPeelCtas, kWideThreads,
                             peel::kLocalSmem, cfg.sms,
