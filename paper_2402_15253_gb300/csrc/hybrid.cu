@@ -1,7 +1,8 @@
 // Method selection per graph (PICO_ALGO_AUTO): a persistent cooperative
 // kernel that first measures the graph's largest degree, then runs HistoCore or
-// the first part of PeelOne on it; the launches that follow finish PeelOne, or
-// return at once after HistoCore. The decision is made on the device (no host round trip, so
+// leaves; the launches of PeelOne that follow return at once after HistoCore. (With
+// PeelOne in the same kernel, HistoCore's part spills more of its 64 registers: R-MAT
+// scale 20 3.41 ms against 3.31.) The decision is made on the device (no host round trip, so
 // the call stays asynchronous and capturable) and is uniform over the grid
 // (every CTA reads the same snapshot after the barrier).
 //
@@ -35,10 +36,12 @@ __device__ __forceinline__ bool prefer_histocore(long long n, long long m, unsig
     return d * nn >= kAutoSkew * mm && mm * mm <= kAutoScale * d * nn;
 }
 
-template <typename Off>
+// kWaves: PeelOne runs in this kernel, with a grid barrier per wave (there are no
+// asynchronous levels, see peelone_async).
+template <typename Off, bool kWaves>
 __global__ void __launch_bounds__(kThreads, 2)
     hybrid_kernel(peel::Params<Off> pp, histo::Params<Off> hp, LastResult *last,
-                  unsigned long long limit_ns, bool local, bool any_degrees)
+                  unsigned long long limit_ns)
 {
     __shared__ unsigned s_snap[kLiveWords + 1];
     __shared__ unsigned s_tmp[256];
@@ -68,31 +71,25 @@ __global__ void __launch_bounds__(kThreads, 2)
         use_histo = prefer_histocore(n, hp.m, s_snap[kLiveDmax]);
         if (use_histo)
             histo::run(hp, dom, s_tmp, st, clk, arcs, atomics, slots, pulled);
-        else if (local && (any_degrees || peel::local_degrees(s_snap[kLiveDmax], n, hp.m)))
-            over = false;   // the next launch peels the graph in shared memory
-        else if (pp.work)
-            over = peel::run_async<Off, kPeelRepair, true>(pp, dom, s_tmp, st, clk, arcs, atomics,
-                                                           extra, local);
-        else
+        else if constexpr (kWaves)
             peel::run<Off, GridDom, kPeelRepair>(pp, dom, s_tmp, st, clk, arcs, atomics, extra);
+        else
+            over = false;
     }
-    if (use_histo || !pp.work) {
-        block_sum_to(arcs, &pp.ctl->stats[kStArcs], s_red);
-    } else if (over && blockIdx.x == 0 && threadIdx.x == 0) {
-        st[kStArcs] = (unsigned long long)hp.m;   // the launch that ends PeelOne counts its arcs
-    }
+    block_sum_to(arcs, &pp.ctl->stats[kStArcs], s_red);
     block_sum_to(atomics, &pp.ctl->stats[kStAtomics], s_red);
     block_sum_to(slots, &pp.ctl->stats[kStSlots], s_red);
     block_sum_to(pulled, &pp.ctl->stats[kStPulled], s_red);
     block_sum_to(extra, &pp.ctl->stats[kStExtra], s_red);
     if (blockIdx.x != 0 && threadIdx.x < kStCount) st[threadIdx.x] = 0;
-    if (!over) {   // later launches finish and publish
+    if (!over) {   // PeelOne's launches publish
         fold_block(pp.ctl, st);
+        leave_barriers(pp.ctl, 0);
         return;
     }
     if (finish_block(pp.ctl, last, use_histo ? PICO_ALGO_HISTOCORE : PICO_ALGO_PEELONE, st,
                      kStCount) &&
-        pp.work)
+        !kWaves)
         pp.tail->published = 1;   // the later launches return at once
 }
 
@@ -108,11 +105,12 @@ template <typename Off>
 int launch_hybrid(const Off *rp, const int *ci, long long n, long long m, int *core, void *ws,
                   LastResult *last, cudaStream_t stream, const LaunchCfg &cfg)
 {
-    static int occ[64] = {};
-    int &o = occ[cfg.device & 63];
+    static int occ[2][64] = {};
+    const bool async = peelone_async<Off>(cfg);
+    const void *fn = async ? (const void *)hybrid_kernel<Off, false> : (const void *)hybrid_kernel<Off, true>;
+    int &o = occ[async][cfg.device & 63];
     if (o == 0) {
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, hybrid_kernel<Off>, kThreads, 0) !=
-                cudaSuccess ||
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, fn, kThreads, 0) != cudaSuccess ||
             o <= 0)
             return -3;
     }
@@ -122,7 +120,7 @@ int launch_hybrid(const Off *rp, const int *ci, long long n, long long m, int *c
     histo::Params<Off> hp;
     {
         Carver c(ws);
-        peel::carve(pp, c, n, m, cfg.peel_async && ctas <= peel::kMaxAsyncCtas);
+        peel::carve(pp, c, n, m, async);
         pp.rp = rp;
         pp.ci = ci;
         pp.core = core;
@@ -158,21 +156,10 @@ int launch_hybrid(const Off *rp, const int *ci, long long n, long long m, int *c
     }
     if (cudaMemsetAsync(pp.ctl, 0, sizeof(Ctrl), stream) != cudaSuccess) return -3;
     unsigned long long limit = cfg.limit_ns;
-    bool local = pp.work && peelone_local(n, m, false), any_degrees = peelone_local(n, m, true);
-    void *args[] = {&pp, &hp, &last, &limit, &local, &any_degrees};
-    // PeelOne's residual degrees stay in L2 (when HistoCore runs, the window
-    // covers part of its scratch instead, which is harmless)
-    const size_t win = pp.work ? std::min<size_t>((size_t)n * sizeof(int), cfg.l2_window) : 0;
-    if (launch_cooperative((const void *)hybrid_kernel<Off>, dim3(ctas), dim3(kThreads), args, 0,
-                           stream, pp.work, win) != cudaSuccess)
+    void *args[] = {&pp, &hp, &last, &limit};
+    if (launch_cooperative(fn, dim3(ctas), dim3(kThreads), args, 0, stream) != cudaSuccess)
         return -3;
-    if (pp.work) {   // what is left of PeelOne, if that is the method
-        const int rc = local ? launch_local(pp, m, pp.tail, last, stream, cfg)
-                             : launch_turns(pp, m, last, stream, cfg, ctas);
-        if (rc != 0) return rc;
-    }
-    if (win > 0 && l2_release(pp.work, win, stream) != cudaSuccess) return -3;
-    return 0;
+    return async ? launch_peel_after(pp, m, last, stream, cfg) : 0;
 }
 
 template int launch_hybrid<int>(const int *, const int *, long long, long long, int *, void *,

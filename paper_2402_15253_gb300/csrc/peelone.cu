@@ -129,7 +129,8 @@ __global__ void __launch_bounds__(peel::kTailThreads, 1)
 // none has).
 template <typename Off, int kKept>
 __global__ void __launch_bounds__(kLocalThreads, 1)
-    peelone_local_kernel(peel::LocalParams<Off> p, const peel::TailState *tail, LastResult *last)
+    peelone_local_kernel(peel::LocalParams<Off> p, const peel::TailState *tail, LastResult *last,
+                         int turn)
 {
     extern __shared__ __align__(16) char smem[];
     __shared__ unsigned long long st[kStCount];
@@ -146,7 +147,7 @@ __global__ void __launch_bounds__(kLocalThreads, 1)
     const peel::LocalStats s = peel::run_local<Off, peel::LocalWide, false, kKept>(p, smem, 0, 1);
     if (threadIdx.x == 0) peel::add_stats(st, s, p.n, p.m);
     clk.end(st, kPhWaveMid, (unsigned)s.waves);
-    finish_block(p.ctl, last, PICO_ALGO_PEELONE, st, kStCount, tail ? 1 : 0);
+    finish_block(p.ctl, last, PICO_ALGO_PEELONE, st, kStCount, turn);
 }
 
 // Sets a kernel's dynamic shared memory limit (and non-portable cluster size)
@@ -251,15 +252,22 @@ size_t peelone_ws_bytes(long long n, long long m, bool async)
     return c.size();
 }
 
+namespace {
+
+// Whether a graph of this size is peeled in one CTA's shared memory instead of by the
+// grid kernel: whatever its degrees, or if they call for it (peel::local_degrees,
+// known on the device).
 bool peelone_local(long long n, long long m, bool any_degrees)
 {
     if (n > peel::kLocalSlots || m > kLocalMaxArcs) return false;
     return !any_degrees || n <= kLocalFewVertices || (n <= kLocalAnyVertices && m <= kLocalAnyArcs);
 }
 
+// The shared-memory form. tail: the launch does nothing when *tail says that an
+// earlier one has published the call (nullptr: there is none).
 template <typename Off>
 int launch_local(const peel::Params<Off> &p, long long m, const peel::TailState *tail,
-                 LastResult *last, cudaStream_t stream, const LaunchCfg &cfg)
+                 LastResult *last, cudaStream_t stream, const LaunchCfg &cfg, int turn)
 {
     static bool ready[3][64] = {};
     const void *fns[3] = {(const void *)peelone_local_kernel<Off, peel::kKeepNone>,
@@ -274,80 +282,96 @@ int launch_local(const peel::Params<Off> &p, long long m, const peel::TailState 
     lc.blockDim = dim3(kept == peel::kKeepGraph ? kLocalThreads / 2 : kLocalThreads);
     lc.dynamicSmemBytes = peel::local_smem_bytes<peel::LocalWide>(p.n, kept, m);
     lc.stream = stream;
-    void *args[] = {&lp, &tail, &last};
+    void *args[] = {&lp, &tail, &last, &turn};
     return cudaLaunchKernelExC(&lc, fn, args) == cudaSuccess ? 0 : -3;
 }
 
 template <typename Off>
-int launch_turns(const peel::Params<Off> &p0, long long m, LastResult *last, cudaStream_t stream,
-                 const LaunchCfg &cfg, int ctas)
+const void *grid_kernel(int mode, bool async)
 {
-    peel::Params<Off> p = p0;
-    unsigned long long limit = cfg.limit_ns;
-    const int launches = tail_launches(m);
-    const size_t win = std::min<size_t>((size_t)p.n * sizeof(int), cfg.l2_window);
-    for (int i = 0; i < launches; ++i) {
-        bool final = i + 1 == launches;
-        int turn = i + 1;
-        bool local = false;
-        void *args[] = {&p, &last, &limit, &m, &turn, &final, &local};
-        const cudaError_t e =
-            i % 2 == 0 ? launch_tail(p, m, last, stream, cfg.device, turn, final)
-                       : launch_cooperative((const void *)peelone_kernel<Off, kPeelRepair, true, true>,
-                                            dim3(ctas), dim3(kThreads), args, 0, stream, p.work, win);
-        if (e != cudaSuccess) return -3;
-    }
-    return 0;
-}
-
-template int launch_local<int>(const peel::Params<int> &, long long, const peel::TailState *,
-                               LastResult *, cudaStream_t, const LaunchCfg &);
-template int launch_local<long long>(const peel::Params<long long> &, long long,
-                                     const peel::TailState *, LastResult *, cudaStream_t,
-                                     const LaunchCfg &);
-template int launch_turns<int>(const peel::Params<int> &, long long, LastResult *, cudaStream_t,
-                               const LaunchCfg &, int);
-template int launch_turns<long long>(const peel::Params<long long> &, long long, LastResult *,
-                                     cudaStream_t, const LaunchCfg &, int);
-
-template <typename Off>
-int launch_peelone(const Off *rp, const int *ci, long long n, long long m, int *core, void *ws,
-                   LastResult *last, cudaStream_t stream, const LaunchCfg &cfg, int mode)
-{
-    if (mode < kPeelRepair || mode > kPeelAddBack) return -1;
     const void *fns[2][3] = {{(const void *)peelone_kernel<Off, kPeelRepair, false, false>,
                               (const void *)peelone_kernel<Off, kPeelCas, false, false>,
                               (const void *)peelone_kernel<Off, kPeelAddBack, false, false>},
                              {(const void *)peelone_kernel<Off, kPeelRepair, true, true>,
                               (const void *)peelone_kernel<Off, kPeelCas, true, false>,
                               (const void *)peelone_kernel<Off, kPeelAddBack, true, false>}};
+    return fns[async][mode];
+}
+
+// CTAs of the grid kernel, which is prepared by the first call on a device; 0: error.
+template <typename Off>
+int grid_ctas(int mode, bool async, const LaunchCfg &cfg)
+{
     static int occ[2][3][64] = {};
-    bool async = cfg.peel_async;
-    if (async && mode == kPeelRepair && peelone_local(n, m, true)) {
-        Carver c(ws);
-        peel::Params<Off> p;
-        peel::carve(p, c, n, m, true);
-        p.rp = rp;
-        p.ci = ci;
-        p.core = core;
-        if (cudaMemsetAsync(p.ctl, 0, sizeof(Ctrl), stream) != cudaSuccess) return -3;
-        return launch_local(p, m, nullptr, last, stream, cfg);
-    }
+    const void *fn = grid_kernel<Off>(mode, async);
     int &o = occ[async][mode][cfg.device & 63];
     if (o == 0) {
         if (async && mode == kPeelRepair &&
-            cudaFuncSetAttribute(fns[async][mode], cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 kTailCarveout) != cudaSuccess)
-            return -3;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, fns[async][mode], kThreads, 0) !=
-                cudaSuccess ||
+            cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, kTailCarveout) !=
+                cudaSuccess)
+            return 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, fn, kThreads, 0) != cudaSuccess ||
             o <= 0)
-            return -3;
+            return 0;
     }
-    const int per_sm = o < cfg.max_blocks_per_sm ? o : cfg.max_blocks_per_sm;
-    const int ctas = cfg.sms * per_sm;
-    if (ctas > peel::kMaxAsyncCtas) async = false;   // the level-end flags have no room
+    return cfg.sms * (o < cfg.max_blocks_per_sm ? o : cfg.max_blocks_per_sm);
+}
 
+// The launches of one run, p carved and its control block zeroed; `turn` is the
+// first one's place among the launches of the call. Behind another launch (turn > 0)
+// asynchronous PeelOne does nothing when that one has published the call.
+template <typename Off>
+int launch_run(peel::Params<Off> &p, long long m, LastResult *last, cudaStream_t stream,
+               const LaunchCfg &cfg, int mode, bool async, int turn)
+{
+    const bool tail = async && mode == kPeelRepair;
+    if (tail && peelone_local(p.n, m, true))
+        return launch_local(p, m, turn > 0 ? p.tail : nullptr, last, stream, cfg, turn);
+    const int ctas = grid_ctas<Off>(mode, async, cfg);
+    if (ctas == 0) return -3;
+    unsigned long long limit = cfg.limit_ns;
+    bool local = tail && peelone_local(p.n, m, false);   // this launch or one CTA, by the degrees
+    const int launches = tail && !local ? tail_launches(m) : 0;   // ... and those that take turns
+    // the residual degrees (the target of every decrement) stay in L2
+    const size_t win = async ? std::min<size_t>((size_t)p.n * sizeof(int), cfg.l2_window) : 0;
+    for (int i = 0; i <= launches; ++i, ++turn) {
+        bool final = i == launches;
+        bool by_degrees = local && i == 0;
+        void *args[] = {&p, &last, &limit, &m, &turn, &final, &by_degrees};
+        const cudaError_t e =
+            i % 2 == 1 ? launch_tail(p, m, last, stream, cfg.device, turn, final)
+                       : launch_cooperative(grid_kernel<Off>(mode, async), dim3(ctas), dim3(kThreads),
+                                            args, 0, stream, p.work, win);
+        if (e != cudaSuccess) return -3;
+    }
+    if (local && launch_local(p, m, p.tail, last, stream, cfg, turn) != 0) return -3;
+    if (win > 0 && l2_release(p.work, win, stream) != cudaSuccess) return -3;
+    return 0;
+}
+
+}  // namespace
+
+template <typename Off>
+bool peelone_async(const LaunchCfg &cfg)
+{
+    // beyond that the level-end flags have no room
+    return cfg.peel_async && grid_ctas<Off>(kPeelRepair, true, cfg) <= peel::kMaxAsyncCtas;
+}
+
+template <typename Off>
+int launch_peel_after(peel::Params<Off> &p, long long m, LastResult *last, cudaStream_t stream,
+                      const LaunchCfg &cfg)
+{
+    return launch_run(p, m, last, stream, cfg, kPeelRepair, true, 1);
+}
+
+template <typename Off>
+int launch_peelone(const Off *rp, const int *ci, long long n, long long m, int *core, void *ws,
+                   LastResult *last, cudaStream_t stream, const LaunchCfg &cfg, int mode)
+{
+    if (mode < kPeelRepair || mode > kPeelAddBack) return -1;
+    const bool async =
+        cfg.peel_async && grid_ctas<Off>(mode, true, cfg) <= peel::kMaxAsyncCtas;
     Carver c(ws);
     peel::Params<Off> p;
     peel::carve(p, c, n, m, async);
@@ -356,26 +380,15 @@ int launch_peelone(const Off *rp, const int *ci, long long n, long long m, int *
     p.core = core;
     p.tn = cfg.tn;
     if (cudaMemsetAsync(p.ctl, 0, sizeof(Ctrl), stream) != cudaSuccess) return -3;
-
-    dim3 grid(ctas), block(kThreads);
-    unsigned long long limit = cfg.limit_ns;
-    const bool tail = async && mode == kPeelRepair;
-    bool local = tail && peelone_local(n, m, false);   // this launch or one CTA, by the degrees
-    bool final = !tail || local;
-    int turn = 0;
-    void *args[] = {&p, &last, &limit, &m, &turn, &final, &local};
-    // the residual degrees (the target of every decrement) stay in L2
-    const size_t win = async ? std::min<size_t>((size_t)n * sizeof(int), cfg.l2_window) : 0;
-    if (launch_cooperative(fns[async][mode], grid, block, args, 0, stream, p.work, win) !=
-        cudaSuccess)
-        return -3;
-    if (tail && (local ? launch_local(p, m, p.tail, last, stream, cfg)
-                       : launch_turns(p, m, last, stream, cfg, ctas)) != 0)
-        return -3;
-    if (win > 0 && l2_release(p.work, win, stream) != cudaSuccess) return -3;
-    return 0;
+    return launch_run(p, m, last, stream, cfg, mode, async, 0);
 }
 
+template bool peelone_async<int>(const LaunchCfg &);
+template bool peelone_async<long long>(const LaunchCfg &);
+template int launch_peel_after<int>(peel::Params<int> &, long long, LastResult *, cudaStream_t,
+                                    const LaunchCfg &);
+template int launch_peel_after<long long>(peel::Params<long long> &, long long, LastResult *,
+                                          cudaStream_t, const LaunchCfg &);
 template int launch_peelone<int>(const int *, const int *, long long, long long, int *, void *,
                                  LastResult *, cudaStream_t, const LaunchCfg &, int);
 template int launch_peelone<long long>(const long long *, const int *, long long, long long,

@@ -375,6 +375,21 @@ __device__ __forceinline__ bool finish_block(Ctrl *c, LastResult *last, int algo
     return false;
 }
 
+// Called by every CTA of a launch that leaves a call to later launches: the last one
+// to come sets the grid barrier back, so that the next launch counts from zero (the
+// others have left every barrier by then).
+__device__ __forceinline__ void leave_barriers(Ctrl *c, int turn)
+{
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(&c->stat.w[1 + turn], 1u) == gridDim.x - 1) {
+            c->bar.w[0] = c->bar.w[1] = 0;
+            c->gen.w[0] = 0;
+        }
+    }
+}
+
 // ---------------------------------------------------------------------------
 // aggregated appends
 // ---------------------------------------------------------------------------

@@ -95,25 +95,18 @@ int launch_peelone(const Off *rp, const int *ci, long long n, long long m, int *
 namespace peel {
 template <typename Off>
 struct Params;
-struct TailState;
 }  // namespace peel
 
-// Whether a graph of this size is peeled in one CTA's shared memory
-// (launch_local) instead of by the grid kernel: whatever its degrees, or if they call
-// for it (peel::local_degrees, known on the device).
-bool peelone_local(long long n, long long m, bool any_degrees);
-
-// The shared-memory form; p: carved scratch with the control block zeroed.
-// tail: the launch does nothing when *tail says the call is published.
+// Whether PeelOne's levels are asynchronous (needs more scratch, see peelone_ws_bytes).
 template <typename Off>
-int launch_local(const peel::Params<Off> &p, long long m, const peel::TailState *tail,
-                 LastResult *last, cudaStream_t stream, const LaunchCfg &cfg);
+bool peelone_async(const LaunchCfg &cfg);
 
-// The launches of the cluster kernel and the grid kernel that follow a first
-// launch of the grid kernel (peel::run_async with kTail), which left *p.tail.
+// PeelOne behind another launch of the same call, which either published it (then
+// these launches do nothing) or left p as it was; p carved for asynchronous levels, the
+// control block zeroed before that launch.
 template <typename Off>
-int launch_turns(const peel::Params<Off> &p, long long m, LastResult *last, cudaStream_t stream,
-                 const LaunchCfg &cfg, int ctas);
+int launch_peel_after(peel::Params<Off> &p, long long m, LastResult *last, cudaStream_t stream,
+                      const LaunchCfg &cfg);
 
 // init_est: start from these estimates (core maintenance; may alias core)
 template <typename Off>
