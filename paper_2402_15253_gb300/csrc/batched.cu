@@ -148,7 +148,8 @@ __device__ __forceinline__ void solve_graph(const BatchParams &bp, int g, Dom &d
         peel::Params<int> p{bp.rp + v0 + g, bp.ci + a0,    n,      bp.core + v0,
                             bp.res0 + v0,   bp.res1 + v0,  bp.qs + v0, chunks,
                             chunk_cap,      bp.ctl,        bp.tn};
-        peel::run(p, dom, s_tmp, st, clk, arcs, atomics, extra);
+        peel::run<int, Dom, kPeelRepair, true>(p, dom, s_tmp, st, clk, arcs, atomics, extra);
+        if (dom.leader()) arcs += (unsigned long long)m;   // every row is expanded once
     } else {
         histo::Params<int> p;
         p.rp = bp.rp + v0 + g;
@@ -298,7 +299,6 @@ __global__ void __launch_bounds__(512, 2) batched_huge_kernel(BatchParams bp)
     }
     block_sum_to(arcs, &bp.ctl->stats[kStArcs], s_red);
     block_sum_to(atomics, &bp.ctl->stats[kStAtomics], s_red);
-    block_sum_to(extra, &bp.ctl->stats[kStExtra], s_red);
     fold_block(bp.ctl, st);
     cluster.sync();   // no CTA leaves while another may still read its shared memory
 }

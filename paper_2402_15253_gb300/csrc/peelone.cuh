@@ -166,7 +166,9 @@ inline void carve(Params<Off> &p, C &c, long long n, long long m, bool async)
     }
 }
 
-template <typename Off, int Mode = kPeelRepair, bool kAsync = false>
+// kLean: only the successful decrements are counted, in one 32-bit word. The three
+// 64-bit counters cost a batch's largest graphs 4 % (registers and adds per arc).
+template <typename Off, int Mode = kPeelRepair, bool kAsync = false, bool kLean = false>
 struct Arc {
     static constexpr int kArcs = 4;
     const Off *rp;
@@ -185,6 +187,7 @@ struct Arc {
     bool hub = false;     // run_async: this walk reads each neighbour before its
                           // decrement (warp-uniform; chunks of high-degree vertices)
     unsigned long long n_arcs = 0, n_atomics = 0, n_extra = 0;
+    unsigned n_lowered = 0;   // kLean
 
     __device__ __forceinline__ bool item(int, int &, int &) { return true; }
 
@@ -209,7 +212,7 @@ struct Arc {
         for (int j = 0; j < kArcs; ++j) {
             old[j] = 0;
             if (valid[j]) {
-                ++n_arcs;
+                if (!kLean) ++n_arcs;
                 if (c[j] > k) {
                     if (Mode == kPeelCas) {   // atomicSub_{>=k}: never below k
                         int cur = c[j];
@@ -229,6 +232,10 @@ struct Arc {
                         }
                     } else {
                         old[j] = atomicSub(core + u[j], 1);
+                        if (kLean) {
+                            n_lowered += old[j] > k;
+                            continue;
+                        }
                         ++n_atomics;
                         if (old[j] <= k) {   // overshoot past k (a racing decrement)
                             if (Mode == kPeelAddBack) {
@@ -297,8 +304,10 @@ __device__ __forceinline__ void repair(const Params<Off> &p, int k, unsigned s0,
 }
 
 // PeelOne on one graph. Every thread of the domain calls it. st: per-CTA
-// statistics in shared memory (thread 0 writes); s_tmp: >= 128 shared words.
-template <typename Off, typename Dom, int Mode = kPeelRepair>
+// statistics in shared memory (thread 0 writes); s_tmp: >= 128 shared words. kLean:
+// `atomics` receives the successful decrements; the arcs (all of them) are the
+// caller's to count.
+template <typename Off, typename Dom, int Mode = kPeelRepair, bool kLean = false>
 __device__ void run(const Params<Off> &p, Dom &dom, unsigned *s_tmp, unsigned long long *st,
                     PhaseClock &clk, unsigned long long &arcs, unsigned long long &atomics,
                     unsigned long long &extra)
@@ -424,12 +433,17 @@ __device__ void run(const Params<Off> &p, Dom &dom, unsigned *s_tmp, unsigned lo
         unsigned s0 = qs0, s1 = qb0;
         while (s0 < e0 || s1 < e1) {
             const unsigned units = (e0 - s0 + 31) / 32 + (e1 - s1);
-            Arc<Off, Mode> f{p.rp, p.core, p.qs, p.qb, p.qb_cap, ctl, live, k, (unsigned)n, p.tn};
+            Arc<Off, Mode, false, kLean> f{p.rp, p.core, p.qs, p.qb, p.qb_cap, ctl, live, k,
+                                          (unsigned)n, p.tn};
             expand(p.rp, p.ci, p.qs + s0, e0 - s0, p.qb + s1, e1 - s1, gwarp, nwarps, f, p.tn,
                    batch_width(e0 - s0, e1 - s1, nwarps));
-            arcs += f.n_arcs;
-            atomics += f.n_atomics;
-            extra += f.n_extra;
+            if (kLean) {
+                atomics += f.n_lowered;
+            } else {
+                arcs += f.n_arcs;
+                atomics += f.n_atomics;
+                extra += f.n_extra;
+            }
             if (!dom.sync()) return;
             if (threadIdx.x == 0) {
                 ++st[kStBarriers];
