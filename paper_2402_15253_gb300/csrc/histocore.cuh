@@ -869,7 +869,9 @@ __device__ void run(const Params<Off> &p0, Dom &dom, unsigned *s_tmp, unsigned l
                     walk_small_batch(p.rp, p.ci, v, f, p.tn.small_deg);
                 } else {
                     const int2 ent = __ldcg(p.ub + (unit - nbatch));   // written by other CTAs
-                    push_chunk(p, ent.x, ent.y, f);
+                    // batches keep no lists
+                    if constexpr (Dom::kGrid) push_chunk(p, ent.x, ent.y, f);
+                    else walk_chunk(p.rp, p.ci, ent.x, ent.y, f, p.tn);
                 }
             }
             arcs += acc.arcs;   // the changed vertices' arcs, as Alg. 6 scans them
