@@ -209,14 +209,18 @@ int validate_impl(const Off *rp, const int32_t *ci, int64_t n, int64_t m, uint32
         cudaGetLastError();
         return PICO_ERR_OOM;
     }
-    unsigned found = 0;
+    const pico::LaunchCfg cfg = cfg_of(d);
+    pico::ValidateWords w{};
+    const auto read = [&] {
+        return cudaMemcpyAsync(&w, flag, sizeof(w), cudaMemcpyDeviceToHost, stream) == cudaSuccess &&
+               cudaStreamSynchronize(stream) == cudaSuccess;
+    };
     bool ok = cudaMemsetAsync(flag, 0, sizeof(*flag), stream) == cudaSuccess &&
-              pico::launch_validate<Off>(rp, ci, n, m, flag, stream, cfg_of(d)) == 0 &&
-              cudaMemcpyAsync(&found, &flag->defects, sizeof(unsigned), cudaMemcpyDeviceToHost,
-                              stream) ==
-                  cudaSuccess;
+              pico::launch_validate<Off>(rp, ci, n, m, flag, stream, cfg) == 0 && read();
+    if (ok && !(w.defects & PICO_DEFECT_ROWS) && (w.suspect || w.excess))
+        ok = pico::launch_validate_exact<Off>(rp, ci, n, flag, stream, cfg) == 0 && read();
     cudaFreeAsync(flag, stream);
-    ok = cudaStreamSynchronize(stream) == cudaSuccess && ok;
+    const uint32_t found = w.defects;
     if (!ok) {
         cudaGetLastError();
         return PICO_ERR_CUDA;

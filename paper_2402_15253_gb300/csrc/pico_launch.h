@@ -148,8 +148,9 @@ int launch_batched(const int64_t *vtx_off, const int64_t *arc_off, int G, const 
 int selftest_handover(LastResult *last, cudaStream_t stream);
 int selftest_wait_timeout(LastResult *last, int limit_ms, cudaStream_t stream, const LaunchCfg &cfg);
 
-// Input validation (validate.cu): ORs the PICO_DEFECT_* bits it finds into
-// words->defects (device memory, zeroed by the caller), stream-ordered.
+// Input validation (validate.cu), stream-ordered; words: device memory, zeroed by the
+// caller. When the rows are in order but `suspect` or `excess` is not zero afterwards,
+// the exact kernel ORs the PICO_DEFECT_* bits of the arcs into words->defects.
 struct ValidateWords {
     unsigned defects;
     unsigned suspect;    // the quick pass found a defect
@@ -158,6 +159,9 @@ struct ValidateWords {
 template <typename Off>
 int launch_validate(const Off *rp, const int *ci, long long n, long long m, ValidateWords *words,
                     cudaStream_t stream, const LaunchCfg &cfg);
+template <typename Off>
+int launch_validate_exact(const Off *rp, const int *ci, long long n, ValidateWords *words,
+                          cudaStream_t stream, const LaunchCfg &cfg);
 
 // The current device's launch configuration and per-device status record
 // (capi.cu); returns a pico_status.

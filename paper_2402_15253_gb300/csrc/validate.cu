@@ -1,7 +1,7 @@
 // Input validation of a single-graph CSR: the paper's graphs are simple and
 // undirected (Sec. II-A), and both methods rely on it (PeelOne decrements
 // each neighbour once per arc, HistoCore's pulled rounds read an edit from
-// the far end of each arc). Three launches on the caller's stream:
+// the far end of each arc). Two launches on the caller's stream, or three:
 //   rows   row_ptr[0] == 0, row_ptr non-decreasing, row_ptr[n] == m;
 //   quick  (only when the rows passed, so that every row lies inside
 //          col_idx) whether every neighbour id is in [0, n), no arc is a
@@ -11,8 +11,8 @@
 //          up there by binary search. In strictly increasing rows two such
 //          arcs never find the same partner, so when all are found and there
 //          are as many of them as of the others, every arc has its reverse.
-//   arcs   (only when the quick pass found something) every arc's defects, each
-//          reverse looked up.
+//   arcs   (only when the quick pass found something, which the host reads) every
+//          arc's defects, each reverse looked up.
 // The quick pass shares the arcs out evenly, up to 512 to a warp: one warp per row
 // leaves a hub's row to a single warp (R-MAT scale 20, n 1.0 M, m 31 M: 9.2 ms).
 // What remains is its gathers: two row bounds per arc, and a lookup in the
@@ -145,12 +145,8 @@ __global__ void __launch_bounds__(256)
 
 template <typename Off>
 __global__ void __launch_bounds__(256)
-    validate_arcs(const Off *rp, const int *ci, long long n, ValidateWords *words)
+    validate_arcs(const Off *rp, const int *ci, long long n, unsigned *flag)
 {
-    // the other kernels ran before on this stream: their words are final here
-    if (words->defects & PICO_DEFECT_ROWS) return;
-    if (words->suspect == 0 && words->excess == 0) return;
-    unsigned *const flag = &words->defects;
     const int lane = threadIdx.x & 31;
     const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
     unsigned bad = 0;
@@ -195,21 +191,32 @@ int launch_validate(const Off *rp, const int *ci, long long n, long long m, Vali
     const int segment =
         (int)std::min<long long>(kSegment, std::max<long long>(32, (m / (8 * most) + 31) & ~31ll));
     const unsigned blocks = (unsigned)std::min<long long>(most, n / 256 + 1);
-    // the exact kernel takes a warp for every row, if it has anything to do
-    const unsigned exact = (unsigned)std::min<long long>(most, n / 8 + 1);
     const unsigned shares = (unsigned)std::min<long long>(most, m / (8 * segment) + 1);
     validate_rows<Off><<<blocks, 256, 0, stream>>>(rp, n, m, &words->defects);
     if (cudaGetLastError() != cudaSuccess) return -3;
     validate_quick<Off><<<shares, 256, 0, stream>>>(rp, ci, n, m, segment, words);
     if (cudaGetLastError() != cudaSuccess) return -3;
-    validate_arcs<Off><<<exact, 256, 0, stream>>>(rp, ci, n, words);
-    if (cudaGetLastError() != cudaSuccess) return -3;
     return 0;
+}
+
+template <typename Off>
+int launch_validate_exact(const Off *rp, const int *ci, long long n, ValidateWords *words,
+                          cudaStream_t stream, const LaunchCfg &cfg)
+{
+    // a warp for every row
+    const long long most = cfg.sms > 0 ? cfg.sms * 8 : 1024;
+    validate_arcs<Off><<<(unsigned)std::min<long long>(most, n / 8 + 1), 256, 0, stream>>>(
+        rp, ci, n, &words->defects);
+    return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
 template int launch_validate<int>(const int *, const int *, long long, long long, ValidateWords *,
                                   cudaStream_t, const LaunchCfg &);
 template int launch_validate<long long>(const long long *, const int *, long long, long long,
                                         ValidateWords *, cudaStream_t, const LaunchCfg &);
+template int launch_validate_exact<int>(const int *, const int *, long long, ValidateWords *,
+                                        cudaStream_t, const LaunchCfg &);
+template int launch_validate_exact<long long>(const long long *, const int *, long long,
+                                              ValidateWords *, cudaStream_t, const LaunchCfg &);
 
 }  // namespace pico
