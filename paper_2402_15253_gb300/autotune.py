@@ -1,16 +1,18 @@
 """Autotuner of the degree-class work assignment.
 
-The kernels assign work by degree class: vertices of degree <= small_deg are
-batched 32 per warp, larger ones are split into chunks of `chunk` arcs (one
-per warp); the batched kernel gives each graph one CTA of `batched_threads`
-threads, or a cluster of 8 CTAs when it has at least 2^cluster_log2 arcs. The
-best values depend on the graph mix and the GPU; results never do. This
+The kernels that work on a graph in global memory assign work by degree class:
+vertices of degree <= small_deg are batched 32 per warp, larger ones are split into
+chunks of `chunk` arcs (one per warp). The batched HistoCore kernel gives each graph
+one CTA of `batched_threads` threads, or a cluster of 8 CTAs when it has at least
+2^cluster_log2 arcs; batched PeelOne chooses its kernels by the graphs' sizes, and of
+these settings only its kernel for graphs above SHARED_VERTICES vertices reads any (the
+first two). The best values depend on the graph mix and the GPU; results never do. This
 module times candidate settings on the caller's own workload (CUDA events on
-the call's stream, median of several runs after a warm-up) in two stages -
-first the degree classes, then the CTA size and cluster threshold - keeps the
-fastest, applies it with pico_set_tuning, and caches it in a JSON file keyed
-by GPU name, method, call kind and power-of-two size classes, so later runs
-of a similar workload start tuned.
+the call's stream, median of several runs after a warm-up) in up to two stages -
+first the degree classes, then the CTA size and cluster threshold, those that the
+workload's kernels read - keeps the fastest, applies it with pico_set_tuning, and
+caches it in a JSON file keyed by GPU name, method, call kind and power-of-two size
+classes, so later runs of a similar workload start tuned.
 
 Cache file: $PICO_TUNING_CACHE, else ~/.cache/pico_gb300/tuning.json.
 """
@@ -28,6 +30,7 @@ CHUNK = (128, 256, 1024)
 THREADS = (256, 512)
 CLUSTER = (21, 23, 62)          # 62: no clusters
 DEFAULT = (32, 256, 512, 21)
+SHARED_VERTICES = 204800        # largest graph that batched PeelOne keeps in shared memory
 
 
 def stages(batched: bool) -> list[list[dict]]:
@@ -38,6 +41,14 @@ def stages(batched: bool) -> list[list[dict]]:
         return [s1]
     s2 = [{"threads": t, "cluster_log2": k} for t in THREADS for k in CLUSTER]
     return [s1, s2]
+
+
+def batched_stages(algo: str, max_vertices: int) -> list[list[dict]]:
+    """The search for a batch whose largest graph has max_vertices vertices: the
+    stages whose settings its kernels read."""
+    if algo == "histocore":
+        return stages(True)
+    return stages(False) if max_vertices > SHARED_VERTICES else []
 
 
 def candidates(batched: bool) -> list[tuple[int, int, int, int]]:
@@ -152,7 +163,8 @@ def _timer(pico, stream, call):
 def tune_batched(pico, vtx_off, arc_off, row_ptr, col_idx, algo="peelone", cands=None,
                  reps: int = 3, use_cache: bool = True, path: str | None = None):
     """Tunes pico_coreness_batched on this packed batch; applies and caches the
-    best setting. Returns (best, timings)."""
+    best setting. A batch that reads none of the settings keeps the current one, which
+    is timed and not cached. Returns (best, timings)."""
     import torch
     a = pico.ALGOS[algo]
     G = vtx_off.numel() - 1
@@ -167,9 +179,15 @@ def tune_batched(pico, vtx_off, arc_off, row_ptr, col_idx, algo="peelone", cands
             raise pico.PicoError(rc, "batched")
 
     run = _timer(pico, stream, call)
-    best, timings = tune(run, cands, reps) if cands else tune_staged(run, stages(True), reps=reps)
+    search = batched_stages(algo, int((vtx_off[1:] - vtx_off[:-1]).max()) if G else 0)
+    if cands:
+        best, timings = tune(run, cands, reps)
+    elif search:
+        best, timings = tune_staged(run, search, reps=reps)
+    else:
+        best, timings = tune(run, [pico.pico_get_tuning()], reps)
     pico.pico_set_tuning(*best)
-    if use_cache:
+    if use_cache and (cands or search):
         key = cache_key(torch.cuda.get_device_name(), algo, "batched", tv, ta, G)
         save_cache({key: list(best)}, path)
     return best, timings

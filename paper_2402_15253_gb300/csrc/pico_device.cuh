@@ -56,7 +56,7 @@ constexpr int kPeelGuard = 4;
 struct Tuning {
     int small_deg;
     int chunk;
-    int cluster_log2;   // batched form: graphs with >= 2^cluster_log2 arcs use a cluster
+    int cluster_log2;   // batched HistoCore: graphs with >= 2^cluster_log2 arcs use a cluster
     int update_mode = kUpdateAuto;
     int pull_pct = kPullPct;
     int peel_guard = kPeelGuard;   // PeelOne: guard the arcs of vertices of degree > peel_guard * k

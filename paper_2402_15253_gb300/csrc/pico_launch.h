@@ -19,7 +19,7 @@ struct LaunchCfg {
     int max_blocks_per_sm;         // cap on co-resident CTAs per SM
     unsigned long long limit_ns;   // time limit of every device-side wait
     Tuning tn;                     // degree-class work assignment
-    int batched_threads;           // threads per CTA of the batched kernel (256 or 512)
+    int batched_threads;           // threads per CTA of the batched HistoCore kernel (256 or 512)
     bool peel_async = false;       // single-graph PeelOne: asynchronous levels (run_async)
     size_t l2_window = 0;          // largest L2 access-policy window to mark persisting (0: none)
     bool validate = false;         // single-graph calls validate their graph first (PICO_VALIDATE=1)
