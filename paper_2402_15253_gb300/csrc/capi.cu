@@ -204,27 +204,32 @@ int validate_impl(const Off *rp, const int32_t *ci, int64_t n, int64_t m, uint32
     DeviceState *d = nullptr;
     int rc = device_state(&d);
     if (rc != PICO_OK) return rc;
-    pico::ValidateWords *flag = nullptr;
-    if (fault_alloc() || cudaMallocAsync(&flag, sizeof(*flag), stream) != cudaSuccess) {
-        cudaGetLastError();
-        return PICO_ERR_OOM;
-    }
     const pico::LaunchCfg cfg = cfg_of(d);
+    // runs `launch` on zeroed words and reads them back; their memory is returned
+    // before the wait, which hides it
     pico::ValidateWords w{};
-    const auto read = [&] {
-        return cudaMemcpyAsync(&w, flag, sizeof(w), cudaMemcpyDeviceToHost, stream) == cudaSuccess &&
-               cudaStreamSynchronize(stream) == cudaSuccess;
+    const auto pass = [&](auto launch) {
+        pico::ValidateWords *words = nullptr;
+        if (fault_alloc() || cudaMallocAsync(&words, sizeof(w), stream) != cudaSuccess) {
+            cudaGetLastError();
+            return (int)PICO_ERR_OOM;
+        }
+        bool ok = cudaMemsetAsync(words, 0, sizeof(w), stream) == cudaSuccess && launch(words) == 0 &&
+                  cudaMemcpyAsync(&w, words, sizeof(w), cudaMemcpyDeviceToHost, stream) == cudaSuccess;
+        cudaFreeAsync(words, stream);
+        ok = cudaStreamSynchronize(stream) == cudaSuccess && ok;
+        if (!ok) cudaGetLastError();
+        return ok ? (int)PICO_OK : (int)PICO_ERR_CUDA;
     };
-    bool ok = cudaMemsetAsync(flag, 0, sizeof(*flag), stream) == cudaSuccess &&
-              pico::launch_validate<Off>(rp, ci, n, m, flag, stream, cfg) == 0 && read();
-    if (ok && !(w.defects & PICO_DEFECT_ROWS) && (w.suspect || w.excess))
-        ok = pico::launch_validate_exact<Off>(rp, ci, n, flag, stream, cfg) == 0 && read();
-    cudaFreeAsync(flag, stream);
+    rc = pass([&](pico::ValidateWords *words) {
+        return pico::launch_validate<Off>(rp, ci, n, m, words, stream, cfg);
+    });
+    if (rc == PICO_OK && !(w.defects & PICO_DEFECT_ROWS) && (w.suspect || w.excess))
+        rc = pass([&](pico::ValidateWords *words) {
+            return pico::launch_validate_exact<Off>(rp, ci, n, words, stream, cfg);
+        });
+    if (rc != PICO_OK) return rc;
     const uint32_t found = w.defects;
-    if (!ok) {
-        cudaGetLastError();
-        return PICO_ERR_CUDA;
-    }
     if (defects) *defects = found;
     return found ? PICO_ERR_BAD_GRAPH : PICO_OK;
 }

@@ -150,7 +150,8 @@ int selftest_wait_timeout(LastResult *last, int limit_ms, cudaStream_t stream, c
 
 // Input validation (validate.cu), stream-ordered; words: device memory, zeroed by the
 // caller. When the rows are in order but `suspect` or `excess` is not zero afterwards,
-// the exact kernel ORs the PICO_DEFECT_* bits of the arcs into words->defects.
+// the exact kernel reports the PICO_DEFECT_* bits of the arcs in words->defects (other
+// words, zeroed as well).
 struct ValidateWords {
     unsigned defects;
     unsigned suspect;    // the quick pass found a defect
