@@ -207,16 +207,11 @@ cudaError_t launch_tail(peel::Params<Off> &p, long long m, LastResult *last, cud
 // and 1.85 with eight. At 5.4 M arcs (scale 17, edge factor 24) one takes 2.06 ms, eight
 // 2.05, and 5.6 M arcs in one heavy level 0.96 and 0.59 (one grid kernel 0.51), hence the
 // line at 4 Mi.
-// Behind the method selection these launches are idle whenever HistoCore was chosen,
-// which it is for most skewed graphs of up to kSelectFew arcs: they get four (R-MAT
-// scale 18, AUTO: 1.63 ms, 1.66 with twelve).
-constexpr int kFewLaunches = 1, kSelectLaunches = 4, kManyLaunches = 12;
-constexpr long long kSelectFew = 40ll << 20;
+constexpr int kFewLaunches = 1, kManyLaunches = 12;
 static_assert(kManyLaunches + 1 < kMaxTurns, "every launch counts its CTAs in a word of its own");
-int tail_launches(long long m, bool selected)
+int tail_launches(long long m)
 {
-    return m < peel::kTailMaxGraph ? kFewLaunches
-                                   : (selected && m < kSelectFew ? kSelectLaunches : kManyLaunches);
+    return m < peel::kTailMaxGraph ? kFewLaunches : kManyLaunches;
 }
 
 // Reads a range (16 bytes a thread per step); the values are not used.
@@ -345,8 +340,7 @@ int launch_run(peel::Params<Off> &p, long long m, LastResult *last, cudaStream_t
     if (ctas == 0) return -3;
     unsigned long long limit = cfg.limit_ns;
     bool local = tail && peelone_local(p.n, m, false);   // this launch or one CTA, by the degrees
-    // ... and those that take turns
-    const int launches = tail && !local ? tail_launches(m, turn > 0) : 0;
+    const int launches = tail && !local ? tail_launches(m) : 0;   // ... and those that take turns
     // the residual degrees (the target of every decrement) stay in L2
     const size_t win = async ? std::min<size_t>((size_t)p.n * sizeof(int), cfg.l2_window) : 0;
     for (int i = 0; i <= launches; ++i, ++turn) {
