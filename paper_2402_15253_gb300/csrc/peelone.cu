@@ -201,13 +201,12 @@ cudaError_t launch_tail(peel::Params<Off> &p, long long m, LastResult *last, cud
 // kernel: 1.17). R-MAT scale 18 and 20 (edge factor 16), 20 (8) and Chung-Lu 2^19 take
 // 2.43, 4.92, 3.63, 4.23 ms with six, 2.44, 4.58, 3.12, 4.12 with eight, 2.46, 4.49,
 // 3.02, 4.14 with twelve launches.
-// Smaller graphs get one launch, on the cluster, which is done with the arcs of a heavy
-// level before the grid would be with the light ones behind it: R-MAT scale 15, 16
-// and 17 1.03, 1.36 and 1.79 ms with one, 1.07, 1.43 and 1.84 with three, 1.07, 1.44
-// and 1.85 with eight. At 5.4 M arcs (scale 17, edge factor 24) one takes 2.06 ms, eight
-// 2.05, and 5.6 M arcs in one heavy level 0.96 and 0.59 (one grid kernel 0.51), hence the
-// line at 4 Mi.
-constexpr int kFewLaunches = 1, kManyLaunches = 12;
+// Smaller graphs end with the cluster kernel, whose light levels at the end cost the
+// grid more than the arcs cost the cluster: R-MAT scale 16 1.36 ms with one launch,
+// 1.43 with four or six, 1.54 with two. One launch alone leaves a graph of 5.6 M arcs
+// behind a single heavy level to the cluster (0.96 ms; one grid kernel 0.51), so they
+// get three.
+constexpr int kFewLaunches = 3, kManyLaunches = 12;
 static_assert(kManyLaunches + 1 < kMaxTurns, "every launch counts its CTAs in a word of its own");
 int tail_launches(long long m)
 {

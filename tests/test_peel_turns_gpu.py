@@ -140,8 +140,9 @@ TURNS = [
     ("wide-wave-with-hub-last", lambda: hub_in_wide_wave(70000, 200000), 1, 0),
     ("spilled-last", lambda: five_tree(60000), 1, 0),
     ("spilled-back", lambda: five_tree(300000), None, 1),
-    # one launch below 4 Mi arcs, on the cluster; twelve above, the last on the grid
-    ("turns-end-on-the-cluster", lambda: alternating(5, 15, 8), 1, 0),
+    # three launches below 6 Mi arcs, the last on the cluster; twelve above, the last
+    # on the grid
+    ("turns-end-on-the-cluster", lambda: alternating(5, 15, 8), 2, 1),
     ("turns-end-on-the-grid", lambda: alternating(8, 37, 25), 6, 6),
 ]
 
