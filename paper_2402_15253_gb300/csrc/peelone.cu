@@ -193,24 +193,16 @@ cudaError_t launch_tail(peel::Params<Off> &p, long long m, LastResult *last, cud
     return cudaLaunchKernelExC(&lc, fn, args);
 }
 
-// Launches that follow the grid kernel's first: cluster and grid kernel in turn. One
-// with nothing to do takes 3.3 us. Graphs of at least kTailMaxGraph arcs get enough
-// for their alternations and end with the grid kernel, since one cluster walks 7 G
-// arcs/s: a graph of 18 M arcs whose alternations run out before them takes 2.72 ms
-// with three launches, the last on the cluster, and 1.13 with twelve (one grid
-// kernel: 1.17). R-MAT scale 18 and 20 (edge factor 16), 20 (8) and Chung-Lu 2^19 take
-// 2.43, 4.92, 3.63, 4.23 ms with six, 2.44, 4.58, 3.12, 4.12 with eight, 2.46, 4.49,
-// 3.02, 4.14 with twelve launches.
-// Smaller graphs end with the cluster kernel, whose light levels at the end cost the
-// grid more than the arcs cost the cluster: R-MAT scale 16 1.36 ms with one launch,
-// 1.43 with four or six, 1.54 with two. One launch alone leaves a graph of 5.6 M arcs
-// behind a single heavy level to the cluster (0.96 ms; one grid kernel 0.51), so they
-// get three.
-constexpr int kFewLaunches = 3, kManyLaunches = 12;
-static_assert(kManyLaunches + 1 < kMaxTurns, "every launch counts its CTAs in a word of its own");
+// Launches that follow the grid kernel's first: cluster and grid kernel in turn.
+// One with nothing to do takes 3.3 us, so small graphs get few and end with the
+// cluster kernel (which walks 5 M arcs at worst in 0.4 ms); large ones end with
+// the grid kernel. R-MAT scales 20 and 21 take 4.75 and 6.20 ms with six, 5.95
+// and 7.22 ms with four.
+constexpr int kMostLaunches = 12;
+static_assert(kMostLaunches < kMaxTurns, "every launch counts its CTAs in a word of its own");
 int tail_launches(long long m)
 {
-    return m < peel::kTailMaxGraph ? kFewLaunches : kManyLaunches;
+    return m < (6 << 20) ? 1 : m < peel::kTailMaxGraph ? 3 : m < (120 << 20) ? 6 : kMostLaunches;
 }
 
 // Reads a range (16 bytes a thread per step); the values are not used.

@@ -94,7 +94,7 @@ constexpr unsigned kTailMaxArcs = 64u << 10;
 constexpr unsigned kTailBudget = 128u << 10;
 // Largest graph whose run may end with a launch of the cluster kernel, which then
 // walks whatever is left.
-constexpr long long kTailMaxGraph = 6ll << 20;
+constexpr long long kTailMaxGraph = 20ll << 20;
 static_assert(sizeof(TailState) <= sizeof(Line), "the control block has no room for TailState");
 constexpr long long kTailSkew = 16;   // largest degree at least this many times the mean
 
