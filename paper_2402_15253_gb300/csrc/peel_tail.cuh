@@ -35,9 +35,9 @@
 //          for itself instead of all.
 //          Vertices that do not fit a queue are listed in global memory and
 //          walked with the next wave.
-//   bail   A wave of more than kTailBudget arcs goes back to the grid kernel,
-//          which finishes the level, unless this is the run's last launch. A
-//          wave of at most kTailThreads vertices is laid out by every CTA, which
+//   bail   A wave of more arcs than the launch's budget goes back to the grid
+//          kernel, which finishes the level, unless this is the run's last launch
+//          (no budget). A wave of at most kTailThreads vertices is laid out by every CTA, which
 //          sees its arcs; those of a wider one are counted first (wave_arcs).
 // The run ends when every vertex is queued: the rest of the last level's walk
 // could only lower vertices that have their coreness.
@@ -56,14 +56,15 @@ constexpr int kTailNear = 8192;          // near-list entries of a CTA
 constexpr int kTailWindow = 32;          // first width of the near window
 
 // A row of d arcs in the sums that a wave is laid out by, which are 32 bits wide
-// (graphs have up to 2^36 arcs). Unless this is the run's last launch, a wave of more
-// than kTailBudget arcs goes back: one row of more is then counted as kTailBudget + 1,
-// and no sum over a tile's 512 rows wraps. The last launch of a run is one of
-// this kernel only for graphs of at most kTailMaxGraph arcs, where nothing wraps.
-__host__ __device__ inline int tail_row(long long d, bool last)
+// (graphs have up to 2^36 arcs). A wave of more than `budget` arcs goes back: a row of
+// more is counted as budget + 1, and no sum over a tile's 512 rows wraps. Without a
+// budget rows count whole, in graphs of at most kTailMaxGraph arcs.
+__host__ __device__ inline int tail_row(long long d, unsigned budget)
 {
-    return last || d <= (long long)kTailBudget ? (int)d : (int)kTailBudget + 1;
+    return d <= (long long)budget ? (int)d : (int)budget + 1;
 }
+static_assert(512ull * (kTailLateBudget + 1) < (1ull << 31) && kTailMaxGraph < kTailNoBudget,
+              "a tile's sum wraps");
 
 struct TailShared {
     long long off[kTailThreads];         // a wave's rows: row start minus position ...
@@ -102,7 +103,7 @@ struct TailPeel {
     TailState *ts;
     TailShared &sh;
     unsigned rank;
-    bool last;   // nothing follows this launch: never bail
+    unsigned budget;   // arcs of a wave that this launch walks, at most
     int k = 0, hi = 0;
     unsigned par = 0, nb = 0, qb = 0;   // exchange parity, near buffer, queue buffer pushed to
     unsigned listed = 0;                // fs entries of the waves so far
@@ -286,7 +287,7 @@ struct TailPeel {
         int d = 0;
         if (v >= 0) {
             rs = p.rp[v];
-            d = tail_row((long long)(p.rp[v + 1] - rs), last);
+            d = tail_row((long long)(p.rp[v + 1] - rs), budget);
         }
         int incl = d;
 #pragma unroll
@@ -295,7 +296,7 @@ struct TailPeel {
             if ((int)lane >= o) incl += y;
         }
         const int total = __shfl_sync(kFull, incl, 31), excl = incl - d;
-        if (!last && (unsigned)total > kTailBudget) return false;
+        if ((unsigned)total > budget) return false;
         const Off off = rs - (Off)excl;
         for (int a0 = (int)(warp * kTailCtas + rank) * 32 * U; a0 < total;
              a0 += (int)nw * kTailCtas * 32 * U) {
@@ -320,8 +321,8 @@ struct TailPeel {
         return true;
     }
 
-    // Arcs of a wave of more than kTailThreads vertices, each CTA's share counted as
-    // at most kTailBudget + 1 per warp (queue not walked yet: qb is the wave's buffer).
+    // Arcs of a wave of more than kTailThreads vertices, counted as at most
+    // budget + 1 per warp (queue not walked yet: qb is the wave's buffer).
     // Without it one CTA would walk a hub in such a wave alone: a wave of 600
     // vertices, one of them with a million leaves, in a graph of 16.4 M arcs, 2.10 ms
     // against 0.84 with it (R-MAT scale 22 and Chung-Lu 2^22 unchanged within 1 %).
@@ -329,15 +330,13 @@ struct TailPeel {
     {
         unsigned sum = 0;
         const auto add = [&](int v) {
-            sum += (unsigned)tail_row((long long)(p.rp[v + 1] - p.rp[v]), false);
+            sum = min(sum + (unsigned)tail_row((long long)(p.rp[v + 1] - p.rp[v]), budget), budget + 1);
         };
-        // at most 8 own vertices a thread and 2^17 / 2^13 listed ones (queued * k is
-        // within the budget), so the sum of a warp does not wrap
         for (unsigned i = threadIdx.x; i < own; i += blockDim.x) add(sh.queue[qb][i]);
         for (unsigned i = rank * blockDim.x + threadIdx.x; i < t.queued - t.fitted;
              i += (unsigned)kTailCtas * blockDim.x)
             add(ldcg(p.fs + listed + i));
-        sum = min(__reduce_add_sync(kFull, sum), kTailBudget + 1);
+        sum = min(__reduce_add_sync(kFull, sum), budget + 1);
         if ((threadIdx.x & 31) == 0 && sum) atomicAdd(&sh.kept, sum);
         return exchange(true).kept;
     }
@@ -358,7 +357,7 @@ struct TailPeel {
             int d = 0;
             if (v >= 0) {
                 rs = p.rp[v];
-                d = tail_row((long long)(p.rp[v + 1] - rs), last);
+                d = tail_row((long long)(p.rp[v + 1] - rs), budget);
             }
             int incl = d;
 #pragma unroll
@@ -376,7 +375,7 @@ struct TailPeel {
             sh.off[tid] = (long long)rs - excl;
             if (tid < 32) sh.start[T + tid] = INT_MAX;
             __syncthreads();
-            if (!last && together && (unsigned)arcs_total > kTailBudget) return false;
+            if (together && (unsigned)arcs_total > budget) return false;
             const int nseg = (arcs_total + 32 * U - 1) / (32 * U);
             const int step = (int)(together ? nw * (unsigned)kTailCtas : nw);
             for (int seg = (int)(together ? warp * (unsigned)kTailCtas + rank : warp); seg < nseg;
@@ -521,8 +520,8 @@ struct TailPeel {
             while (t.queued > 0 && left > 0) {
                 const unsigned b = qb, own = min(sh.x[par ^ 1u][rank][0].x, (unsigned)kTailQueue);
                 settle(b, own);
-                if (!last && ((unsigned long long)t.queued * (unsigned)k > kTailBudget ||
-                              (t.queued > T && wave_arcs(t, own) > kTailBudget))) {
+                if ((unsigned long long)t.queued * (unsigned)k > budget ||
+                    (budget != kTailNoBudget && t.queued > T && wave_arcs(t, own) > budget)) {
                     mode = kTailPending;
                 } else {
                     qb ^= 1u;

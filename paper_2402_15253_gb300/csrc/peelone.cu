@@ -92,7 +92,8 @@ __global__ void __launch_bounds__(kThreads, 2)
 // kernel (peel_tail.cuh).
 template <typename Off>
 __global__ void __launch_bounds__(peel::kTailThreads, 1)
-    peelone_tail_kernel(peel::Params<Off> p, LastResult *last, long long m, int turn, bool final)
+    peelone_tail_kernel(peel::Params<Off> p, LastResult *last, long long m, int turn,
+                        unsigned budget)
 {
     extern __shared__ __align__(16) char smem[];
     __shared__ unsigned long long st[kStCount];
@@ -100,6 +101,7 @@ __global__ void __launch_bounds__(peel::kTailThreads, 1)
     // nothing to do (the same in every CTA)
     if (p.tail->published) return;
     const bool failed = status_of(p.ctl) != 0;
+    const bool final = budget == peel::kTailNoBudget;   // the run's last launch
     if (!final && (p.tail->mode != peel::kTailScan || failed)) return;
     if (threadIdx.x < kStCount) st[threadIdx.x] = 0;
     PhaseClock clk;
@@ -110,7 +112,7 @@ __global__ void __launch_bounds__(peel::kTailThreads, 1)
     __syncthreads();
     clk.start();
     peel::TailPeel<Off> tp{p, p.tail, *reinterpret_cast<peel::TailShared *>(smem), blockIdx.x,
-                            final};
+                            budget};
     const bool over = failed || tp.run(st);
     if (over && blockIdx.x == 0 && threadIdx.x == 0) st[kStArcs] = (unsigned long long)m;
     clk.end(st, kPhWaveMid, (unsigned)st[kStLevels]);
@@ -167,7 +169,7 @@ bool prepare_kernel(const void *fn, size_t smem, bool wide_cluster, bool &ready)
 
 template <typename Off>
 cudaError_t launch_tail(peel::Params<Off> &p, long long m, LastResult *last, cudaStream_t stream,
-                        int device, int turn, bool final)
+                        int device, int turn, unsigned budget)
 {
     static bool ready[64] = {};
     const void *fn = (const void *)peelone_tail_kernel<Off>;
@@ -189,20 +191,35 @@ cudaError_t launch_tail(peel::Params<Off> &p, long long m, LastResult *last, cud
     lc.stream = stream;
     lc.attrs = attr;
     lc.numAttrs = 1;
-    void *args[] = {&p, &last, &m, &turn, &final};
+    void *args[] = {&p, &last, &m, &turn, &budget};
     return cudaLaunchKernelExC(&lc, fn, args);
 }
 
-// Launches that follow the grid kernel's first: cluster and grid kernel in turn.
-// One with nothing to do takes 3.3 us, so small graphs get few and end with the
-// cluster kernel (which walks 5 M arcs at worst in 0.4 ms); large ones end with
-// the grid kernel. R-MAT scales 20 and 21 take 4.75 and 6.20 ms with six, 5.95
-// and 7.22 ms with four.
+// Launches that follow the grid kernel's first: cluster and grid kernel in turn. One
+// with nothing to do takes 3.3 us, so small graphs get few. The cluster walks 7 G
+// arcs/s, a fifth of what the grid does; the grid takes 17 us for a light level, the
+// cluster 6. So what the last launches are left with decides:
+//   below 6 Mi arcs one launch, on the cluster, which walks whatever is left. R-MAT
+//   scale 16: 1.36 ms, 1.39 with a launch of the grid behind it; at worst, 5.6 M arcs
+//   behind one heavy level, 0.96 ms (0.84 with it; one grid kernel 0.51).
+//   below 20 Mi four; the second of the cluster keeps waves of up to 1 M arcs. R-MAT
+//   scale 18, 19 and scale 20 with edge factor 8: 2.57, 3.20, 3.20 ms, with waves of
+//   128 K 2.52, 3.15, 4.36, with three launches 2.57, 3.38, 3.31; 18 M arcs behind two
+//   heavy levels 1.30 ms, with three launches 2.66 (one grid kernel 1.17).
+//   then six, from 120 Mi twelve: R-MAT scale 20 takes 4.75 ms with six, 5.95 with four.
 constexpr int kMostLaunches = 12;
-static_assert(kMostLaunches < kMaxTurns, "every launch counts its CTAs in a word of its own");
+static_assert(kMostLaunches + 1 < kMaxTurns, "every launch counts its CTAs in a word of its own");
+constexpr long long kFourLaunches = 20ll << 20;
 int tail_launches(long long m)
 {
-    return m < (6 << 20) ? 1 : m < peel::kTailMaxGraph ? 3 : m < (120 << 20) ? 6 : kMostLaunches;
+    return m < peel::kTailMaxGraph ? 1 : m < kFourLaunches ? 4 : m < (120 << 20) ? 6 : kMostLaunches;
+}
+
+// Arcs of a wave that the cluster kernel's launch i walks at most.
+unsigned tail_budget(long long m, int i)
+{
+    if (m < peel::kTailMaxGraph) return peel::kTailNoBudget;
+    return m < kFourLaunches && i == 3 ? peel::kTailLateBudget : peel::kTailBudget;
 }
 
 // Reads a range (16 bytes a thread per step); the values are not used.
@@ -339,7 +356,7 @@ int launch_run(peel::Params<Off> &p, long long m, LastResult *last, cudaStream_t
         bool by_degrees = local && i == 0;
         void *args[] = {&p, &last, &limit, &m, &turn, &final, &by_degrees};
         const cudaError_t e =
-            i % 2 == 1 ? launch_tail(p, m, last, stream, cfg.device, turn, final)
+            i % 2 == 1 ? launch_tail(p, m, last, stream, cfg.device, turn, tail_budget(m, i))
                        : launch_cooperative(grid_kernel<Off>(mode, async), dim3(ctas), dim3(kThreads),
                                             args, 0, stream, p.work, win);
         if (e != cudaSuccess) return -3;

@@ -92,9 +92,11 @@ struct TailState {
 constexpr unsigned kTailMaxResidual = 512u << 10;
 constexpr unsigned kTailMaxArcs = 64u << 10;
 constexpr unsigned kTailBudget = 128u << 10;
-// Largest graph whose run may end with a launch of the cluster kernel, which then
-// walks whatever is left.
-constexpr long long kTailMaxGraph = 20ll << 20;
+// The budgets of the cluster kernel's last launch, by the size of the graph (see
+// tail_launches): as any other, wider, or none, when no launch of the grid follows.
+constexpr unsigned kTailLateBudget = 1u << 20;
+constexpr unsigned kTailNoBudget = 0x7ffffffe;
+constexpr long long kTailMaxGraph = 6ll << 20;   // largest graph that goes without
 static_assert(sizeof(TailState) <= sizeof(Line), "the control block has no room for TailState");
 constexpr long long kTailSkew = 16;   // largest degree at least this many times the mean
 

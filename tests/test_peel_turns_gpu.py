@@ -122,12 +122,12 @@ def five_tree(core):
     return union(first[7] + size[7], *pairs)
 
 
-def alternating(parts):
+def alternating(parts, first, step):
     """Heavy levels (9,000 vertices of a complete bipartite part each) with light
     ones between them, next to a star."""
     graphs = [gg.star_graph(90000)]
     for i in range(parts):
-        k = 37 + 25 * i
+        k = first + step * i
         left = torch.arange(k).repeat_interleave(9000)
         graphs += [gg.csr_from_pairs(left, k + torch.arange(9000).repeat(k), k + 9000),
                    gg.complete_graph(k + 6)]
@@ -140,8 +140,12 @@ TURNS = [
     ("wide-wave-with-hub-last", lambda: hub_in_wide_wave(70000, 200000), 1, 0),
     ("spilled-last", lambda: five_tree(60000), 1, 0),
     ("spilled-back", lambda: five_tree(300000), None, 1),
-    ("turns-end-on-the-cluster", lambda: alternating(7), 2, 1),
-    ("turns-end-on-the-grid", lambda: alternating(10), 3, 3),
+    # one launch below 6 Mi arcs, on the cluster; four below 20 Mi (the second of the
+    # cluster walks these heavy levels), then six: the last on the grid
+    ("turns-end-on-the-cluster", lambda: alternating(5, 15, 8), 1, 0),
+    ("four-turns", lambda: alternating(7, 37, 13), 2, 1),
+    ("turns-end-on-the-grid", lambda: alternating(10, 37, 25), 3, 3),
+    ("late-budget", lambda: alternating(3, 37, 80), 2, 2),
 ]
 
 

@@ -18,11 +18,11 @@ PROGRAM = r"""
 using namespace pico::peel;
 int main()
 {
-    const long long lengths[] = {1, 129, kTailBudget - 1, kTailBudget, kTailBudget + 1, 125000000,
-                                 1073741824, 2147483646};
     const int rows[] = {1, 2, 3, 4, 17, 35, 512};
     int bad = 0;
-    for (long long d : lengths)
+    for (unsigned budget : {kTailBudget, kTailLateBudget})
+    for (long long d : {1ll, 129ll, (long long)budget - 1, (long long)budget, (long long)budget + 1,
+                        125000000ll, 1073741824ll, 2147483646ll})
         for (int n : rows)
             for (long long other : {1ll, 4194304ll}) {
                 // n rows of d arcs and 512 - n of `other`, summed as a tile is
@@ -31,14 +31,14 @@ int main()
                 for (int i = 0; i < 512; ++i) {
                     const long long x = i < n ? d : other;
                     exact += x;
-                    sum = (int)((unsigned)sum + (unsigned)tail_row(x, false));
+                    sum = (int)((unsigned)sum + (unsigned)tail_row(x, budget));
                     bad += sum < 0;
                 }
-                bad += ((unsigned)sum > kTailBudget) != (exact > (long long)kTailBudget);
-                if (exact <= (long long)kTailBudget) bad += sum != exact;
+                bad += ((unsigned)sum > budget) != (exact > (long long)budget);
+                if (exact <= (long long)budget) bad += sum != exact;
             }
-    // the last launch counts rows whole, in graphs whose arcs fit 32 bits
-    bad += tail_row(kTailMaxGraph, true) != kTailMaxGraph || kTailMaxGraph >= (1ll << 31);
+    // without a budget rows count whole, in graphs whose arcs fit 32 bits
+    bad += tail_row(kTailMaxGraph, kTailNoBudget) != kTailMaxGraph;
     printf("bad %d\n", bad);
     return bad != 0;
 }
