@@ -69,7 +69,7 @@ def peaks():
 
 
 KERNEL_SOURCES = {
-    "peelone": ("pico_device.cuh", "peelone.cuh", "peelone.cu"),
+    "peelone": ("pico_device.cuh", "peelone.cuh", "peel_tail.cuh", "peelone.cu"),
     "histocore": ("pico_device.cuh", "histocore.cuh", "histocore.cu"),
 }
 

@@ -17,8 +17,9 @@
 // Middle and large graphs share one launch: clusters first take the large
 // graphs, then each CTA takes middle ones. It does not wait for the launch of
 // the huge graphs before it, which leaves SMs free (24 graphs of 1 M vertices and
-// 488 smaller ones: 27.2 ms one after the other, 23.7 ms side by side). The tiny
-// graphs are the last launch, which waits for both.
+// 488 smaller ones, 1.2 G arcs: 28.6 ms one after the other, 25.6 ms side by side). The
+// tiny graphs are the last launch, which waits for both (2,000 of them behind one graph
+// of 1 M vertices add 0.3 ms).
 //
 // HistoCore runs the single-graph body (histo::run) in two phases: graphs of
 // at least 2^cluster_log2 arcs (a tuning value) by clusters of kClusterCtas
@@ -260,12 +261,13 @@ __device__ __forceinline__ peel::LocalParams<int> local_params(const BatchParams
 // PeelOne, huge graphs: one cluster per graph. Bound by the latency of L2 atomics
 // and of the cluster barriers; 8 CTAs of 512 threads, two to an SM, keep twice the
 // warps that 4 CTAs of 1,024 have, and leave room for a second graph beside them
-// (one R-MAT graph of 2^20 vertices and 31 M arcs: 35 ms with those, 15.9 ms so; 24 of them
-// and 488 smaller graphs: 41.8 and 24.4 ms).
+// (one R-MAT graph of 2^20 vertices and 31 M arcs: 35 ms with those, 15.7 ms so; 24 of them
+// and 488 smaller graphs: 41.8 and 25.6 ms).
 // Its reads of residual degrees hit in L1, so it prefers all of an SM's memory as L1.
 // Without that preference it starts on the SMs that another stream's wide CTAs
 // have left with 28 KB of L1, and takes 43 ms instead of 21 (two or four streams of
-// such batches: 35.7 ms a batch, 22.4 with it, 25.4 with one kernel for all classes).
+// such batches: 35.7 ms a batch, 22.4 with it, 25.4 with one kernel for all classes; 21.5
+// since the tickets below).
 __global__ void __launch_bounds__(512, 2) batched_huge_kernel(BatchParams bp)
 {
     namespace cg = cooperative_groups;
@@ -359,8 +361,8 @@ __global__ void __launch_bounds__(kWideThreads, 1) batched_peel_kernel(BatchPara
     if (blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-// PeelOne, tiny graphs; the second launch of a batch, which publishes its
-// status and statistics.
+// PeelOne, tiny graphs; the last launch of a batch, which publishes its status and
+// statistics.
 __global__ void __launch_bounds__(kTinyThreads, 8) batched_tiny_kernel(BatchParams bp, LastResult *last)
 {
     extern __shared__ __align__(16) char smem[];

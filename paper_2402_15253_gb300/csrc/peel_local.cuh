@@ -5,9 +5,9 @@
 // differs is where the decrements go. In global memory every decrement is an
 // L2 round trip, and L2 serves 0.56 returning atomics per clock and SM when
 // every SM issues them (measured, random words of 16 MB); shared memory
-// serves at least 7 per clock and SM, 42 clocks each instead of 515. So each
-// CTA keeps the residual degrees of the vertices it owns in shared memory,
-// needs no guard read before a decrement (a decrement of a queued vertex
+// serves at least 7 per clock and SM, 42 clocks each in a chain of one warp where L2
+// takes 720. So each CTA keeps the residual degrees of the vertices it owns in shared
+// memory, needs no guard read before a decrement (a decrement of a queued vertex
 // returns at most k and is ignored), and a wave ends with __syncthreads.
 //
 //   one CTA    (n <= kLocalSlots) owns every vertex.
@@ -89,7 +89,8 @@ struct LocalStats {
 // What a CTA that peels a graph alone keeps of it in shared memory besides the
 // residual degrees: the row offsets, or all of it. A wave of a small graph is a
 // chain of dependent accesses (row bounds, columns, decrements), and each of
-// the first two takes some 500 clocks from L2 and 30 from shared memory.
+// the first two takes some 500 clocks from L2 (440-535, a load of one warp) and 30 from
+// shared memory.
 enum : int { kKeepNone = 0, kKeepRows = 1, kKeepGraph = 2 };
 
 // Dynamic shared memory of a CTA that owns `n` vertices (and the m arcs of the

@@ -11,8 +11,9 @@
 // left, and those with nothing to do return at once.
 //
 // Residual degrees stay in global memory, where the grid kernel needs them: L2
-// serves a cluster of 16 SMs 0.83 returning atomics per clock and SM with a
-// latency of 515 clocks, distributed shared memory 0.32 with 247 (measured).
+// serves a cluster of 16 SMs 0.83 returning atomics per clock and SM, distributed
+// shared memory 0.32; one warp's chain of them takes 720 and 247 clocks each (measured,
+// words that L2 holds).
 //
 // A level:
 //   scan   Each CTA keeps its own part of the residual list (in global memory)
@@ -149,8 +150,7 @@ struct TailPeel {
 
     // Queues vertices at level k. Their coreness is written at the start of the
     // wave that walks them (settle): stores still in flight would hold up the
-    // cluster barrier (985 clocks instead of 450). What does not fit is listed in global memory
-    // (not during a scan, which the grid kernel then repeats).
+    // cluster barrier (985 clocks instead of 450). What does not fit is listed in global memory.
     template <int N>
     __device__ __forceinline__ void push(const bool (&in)[N], const int (&v)[N])
     {

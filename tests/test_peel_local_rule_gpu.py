@@ -54,3 +54,38 @@ def test_form(pico, name, make, one_cta, off):
             assert st["atomics"] - st["extra"] == ost["decrements"]
         else:
             assert algo == "auto"
+
+
+_CHILD = r"""
+import sys
+import numpy as np
+import torch
+sys.path.insert(0, sys.argv[1])
+import graphgen as gg
+import oracle
+import paper_2402_15253_gb300 as pico
+torch.cuda.set_device(0)
+algos = set()
+for g in (gg.er_graph(30000, 90000, 1), gg.rmat_graph(14, 12, 2), gg.star_graph(40000),
+          gg.grid_graph(60, 70)):
+    want = oracle.bz_coreness(*g.numpy())
+    for off in (torch.int32, torch.int64):
+        got = pico.coreness(g.row_ptr.to("cuda", dtype=off), g.col_idx.cuda(), "auto")
+        assert np.array_equal(got.cpu().numpy(), want)
+        algos.add(pico.pico_get_stats()["algo"])
+print("RESULT", sorted(algos))
+"""
+
+
+@pytest.mark.parametrize("waves", ["0", "1"])
+def test_selection_with_and_without_asynchronous_levels(pico, waves):
+    """AUTO by either form of PeelOne: PICO_PEEL_WAVES=1 keeps it in the selection's
+    own kernel. Both methods are chosen for some graph."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", _CHILD, root], capture_output=True, text=True,
+                       env=dict(os.environ, PICO_PEEL_WAVES=waves), timeout=300)
+    assert r.returncode == 0, r.stderr
+    assert r.stdout.strip().splitlines()[-1] == "RESULT [0, 1]"
