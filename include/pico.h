@@ -138,7 +138,7 @@ int pico_validate_graph_i64(const int64_t *row_ptr, const int32_t *col_idx, int6
                             uint32_t *defects, pico_stream_t stream);
 
 /*
- * Coreness of G independent graphs packed back to back, in one launch.
+ * Coreness of G independent graphs packed back to back, in one call.
  * Coreness is defined per graph (Sec. I), so the result equals G separate
  * calls; each graph must satisfy the single-graph contract and may be empty.
  *   vtx_off, arc_off: device int64 prefix offsets, G + 1 entries each
